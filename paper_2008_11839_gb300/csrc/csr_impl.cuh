@@ -379,18 +379,18 @@ static gconn_status static_run(uint32_t n, uint64_t m, const uint32_t* edges, co
     }
     L2Window l2win;
     l2win.apply(st, P, sizeof(uint32_t) * (size_t)n);
-    if (!csr) GC_TRY(init_state(s, st));   // csr_connect initialises P and its counters
+    bool finalized = false;
+    if (!csr && !finalized) GC_TRY(init_state(s, st));   // csr_connect initialises P and its counters
     if (csr && want_forest)
         GC_TRY(launch("check_arcs", k_check_arcs<OffT>, 1, 1, 0, st, d_off, n, s.err));
 
-    if (!csr) {
+    if (!csr && !finalized) {
         if (is_rounds_link(v.link)) {
             GC_TRY(rounds_coo(v, s, d_edges, nullptr, m, st));
         } else {
-            GC_TRY(union_coo(v, s, d_edges, m, 0, st));
+            GC_TRY(union_coo_static(v, s, d_edges, m, st));
         }
     }
-    bool finalized = false;
     if (csr) GC_TRY(csr_connect(v, s, d_off, d_cols, st, nullptr, labels ? &finalized : nullptr));
     if (labels) {
         // rounds-based finishes leave P fully compressed and min-rooted

@@ -332,7 +332,7 @@ static gconn_status enqueue_batch(gconn_batch* b, cudaStream_t st) {
             uint64_t m = b->heo[g + 1] - b->heo[g];
             UFState s = make_state(n, b->labels + b->hvo[g], nullptr, nullptr, nullptr, v);
             GC_TRY(init_state(s, st));
-            GC_TRY(union_coo(v, s, b->edges + 2 * b->heo[g], m, 0, st));
+            GC_TRY(union_coo_static(v, s, b->edges + 2 * b->heo[g], m, st));
             GC_TRY(finalize_labels(v, s, s.P, st));
         }
     }

@@ -1,0 +1,78 @@
+// gconn_coo.cu -- the union-find finish over a COO edge list: static passes
+// (Algorithm 1 on COO input, Section 2) and insert batches (Section 3.5).
+#include <cuda_runtime.h>
+#include <stdint.h>
+
+#include <algorithm>
+
+#include "csr_impl.cuh"
+#include "gc_internal.h"
+#include "gc_static.h"
+#include "static_kernels.cuh"
+
+namespace gc {
+
+gconn_status union_coo(const Variant& v, const UFState& s, const uint32_t* edges, uint64_t m,
+                       uint32_t eid_base, cudaStream_t st) {
+    if (m == 0) return GCONN_OK;
+    int L, F, S;
+    uf_triple(v, &L, &F, &S);
+    int B = block_of(v);
+    return dispatch_uf(L, F, S, s.sf != nullptr, [&]<int l, int f, int sp, bool sf>() {
+        auto k = k_union_coo<l, f, sp, sf>;
+        // at most about one thread per vertex: beyond that, concurrent unions
+        // on a small vertex set mostly contend for the same few roots (ER
+        // n = 65,536, m = 2^20, Rem-CAS + splice: 0.140 ms with the full
+        // grid, 0.097 ms with a quarter of it, 0.116 ms with an eighth)
+        uint64_t gr = grid_for(k, B, m);
+        const uint64_t cap = std::max<uint64_t>((uint64_t)num_sms(), ((uint64_t)s.n + B - 1) / B);
+        return launch_pdl("union_coo", k, (unsigned)std::min(gr, cap), B, 0, st, (const uint2*)edges, m, s, eid_base);
+    });
+}
+
+// The COO finish of a static pass (every vertex a singleton at the start).
+// Three forms, by size:
+// - fewer edges than fill the GPU once (m < 49,152): one union per thread;
+//   comparing first only adds a round trip (ER n = 16,000, m = 32,000: 34 against
+//   53 us).
+// - 2^15 <= n <= 2^19 and m >= 2n: as many threads as vertices or more would
+//   start on singletons at once and contend for the same few roots.  So about
+//   3n/4 edges, spread over the list, are united first (where a random graph's
+//   giant component appears), the trees are flattened, and the other edges then
+//   mostly find equal parents.  ER n = 65,536, m = 2^20: 98 -> 49 us (85 without
+//   the first pass; a sample of n/2 or n edges 80, 50); n = 200,000, m = 16n:
+//   168 -> 80 (98); RMAT n = 400,000, m = 8n: 144 -> 82 (84).  Above 2^19 the
+//   first wave no longer covers the vertices (RMAT n = 10^6: 156 us without,
+//   173 with); at 16,000 vertices the two launches cost what they save (45, 48).
+// - otherwise one pass over all edges.
+gconn_status union_coo_static(const Variant& v, const UFState& s, const uint32_t* edges, uint64_t m, cudaStream_t st) {
+    if (v.link == GCONN_LINK_JTB || m < 49152) return union_coo(v, s, edges, m, 0, st);
+    int L, F, S;
+    uf_triple(v, &L, &F, &S);
+    const int B = block_of(v);
+    const uint64_t n = s.n;
+    return dispatch_uf(L, F, S, s.sf != nullptr, [&]<int l, int f, int sp, bool sf>() -> gconn_status {
+        if constexpr (l == LK_JTB) return GCONN_E_UNSUPPORTED;   // handled above
+        else {
+            auto pass = [&](const char* name, bool dense, CooPart part, uint64_t count) {
+                auto k = dense ? k_union_filter<l, f, sp, sf, 8> : k_union_filter<l, f, sp, sf, 2>;
+                return launch_pdl(name, k, grid_for(k, B, count / (dense ? 8 : 2) + 1), B, 0, st, (const uint2*)edges,
+                                  m, s, part);
+            };
+            const bool dense = m >= 4 * n;   // most edges join nothing
+            // rules that compress nothing on the way (naive finds of
+            // Union-Async and Union-Hooks, Afforest)
+            constexpr bool bare = f == FD_NAIVE && (l == LK_ASYNC || l == LK_HOOKS || l == LK_AFFOREST);
+            if (bare && n < (1u << 15)) return union_coo(v, s, edges, m, 0, st);
+            if (n >= (1u << 15) && (bare || n <= (1u << 19)) && m >= 2 * n) {
+                const uint32_t every = (uint32_t)std::min<uint64_t>(4 * m / (3 * n), 1u << 30);
+                GC_TRY(pass("union_coo_sample", false, CooPart{COO_SAMPLE, every}, m / every + 32));
+                GC_TRY(finalize_labels(v, s, s.P, st));
+                return pass("union_coo", dense, CooPart{COO_REST, every}, m);
+            }
+            return pass("union_coo", dense, CooPart{COO_ALL, 0}, m);
+        }
+    });
+}
+
+}  // namespace gc

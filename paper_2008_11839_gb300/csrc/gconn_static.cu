@@ -48,24 +48,6 @@ gconn_status init_state(const UFState& s, cudaStream_t st, uint32_t* zero, uint3
     return launch_pdl("init", k_init, grid_for(k_init, 256, s.n), 256, 0, st, s.n, s.P, s.H, s.W, s.sf, zero, nzero);
 }
 
-gconn_status union_coo(const Variant& v, const UFState& s, const uint32_t* edges, uint64_t m,
-                       uint32_t eid_base, cudaStream_t st) {
-    if (m == 0) return GCONN_OK;
-    int L, F, S;
-    uf_triple(v, &L, &F, &S);
-    int B = block_of(v);
-    return dispatch_uf(L, F, S, s.sf != nullptr, [&]<int l, int f, int sp, bool sf>() {
-        auto k = k_union_coo<l, f, sp, sf>;
-        // at most about one thread per vertex: beyond that, concurrent unions
-        // on a small vertex set mostly contend for the same few roots (ER
-        // n = 65,536, m = 2^20, Rem-CAS + splice: 0.140 ms with the full
-        // grid, 0.097 ms with a quarter of it, 0.116 ms with an eighth)
-        uint64_t gr = grid_for(k, B, m);
-        const uint64_t cap = std::max<uint64_t>((uint64_t)num_sms(), ((uint64_t)s.n + B - 1) / B);
-        return launch("union_coo", k, (unsigned)std::min(gr, cap), B, 0, st, (const uint2*)edges, m, s, eid_base);
-    });
-}
-
 gconn_status compress_all(const Variant& v, const UFState& s, cudaStream_t st) {
     if (s.n == 0) return GCONN_OK;
     if (v.link == GCONN_LINK_JTB)

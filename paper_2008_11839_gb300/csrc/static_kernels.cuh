@@ -67,12 +67,13 @@ static __global__ void k_init(uint32_t n, uint32_t* P, uint32_t* H, u64w* W, uin
     }
 }
 
-// Finish phase over a COO edge list (Section 3.5 batches use it too): one
-// union per edge, grid-stride, edges streamed once.  eid_base offsets the
-// recorded forest ids (incremental batches).
+// Insert batches (Section 3.5), and Union-JTB's COO finish: one union per
+// edge, grid-stride, edges streamed once.  eid_base offsets the recorded
+// forest ids.
 template <int L, int F, int S, bool SF>
 static __global__ void __launch_bounds__(256) k_union_coo(const uint2* __restrict__ E, uint64_t m, UFState s,
                                                    uint32_t eid_base) {
+    pdl_entry();
     uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
     uint32_t it = 0;
     for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < m; i += stride) {
@@ -86,6 +87,93 @@ static __global__ void __launch_bounds__(256) k_union_coo(const uint2* __restric
         Spin sp(s.cap);
         uf_union<L, F, S, SF>(s, e.x, e.y, eid_base + (uint32_t)i, sp);
     }
+}
+
+// Which edges a union pass over a COO list takes, in chunks of 32 edges:
+// every chunk, one chunk in `every` (spread over the whole list, so that an
+// ordered list is sampled evenly too), or the chunks that pass left out.
+enum { COO_ALL = 0, COO_SAMPLE = 1, COO_REST = 2 };
+struct CooPart {
+    int mode;
+    uint32_t every;
+};
+
+// Finish phase over a static COO list, for lists where most edges join nothing
+// or climbs are uneven: a warp loads ILP chunks of 32 edges, compares the
+// parents of all of them (ILP x 2 independent gathers in flight; equal parents,
+// even stale ones, mean the same set), packs the edges that differ into a queue
+// and runs their unions 32 at a time with full lanes.
+// The bound is the SM's L1-miss path: random 4-byte loads that miss L1 run at
+// one lane per clock per SM (312 G/s measured, whatever the occupancy and up
+// to 64 MB of P), and an edge needs two.  RMAT n = 2^22, m = 2^26: 1,308 us with
+// a union per thread (k_union_coo), 530 us here, of which the two gathers an
+// edge account for 430 us.  RMAT n = 10^6, m = 1.6 x 10^7: 294 -> 156 us;
+// 4096 x 4096 grid + 64 paths of 2^18 (m = 1.45 n): 2,796 -> 2,182 us.
+// ILP by density: where most edges link (m < 4n) the compared parents are used
+// again by the union, and more edges in flight only push them out of L1 (grid +
+// paths: 2,182, 2,499, 2,803 us with 2, 4, 8); dense lists want the loads in
+// flight (RMAT n = 2^22: 571, 546, 530 us).  A queue of more than 64 entries a
+// warp costs more L1 than it saves (RMAT n = 2^22: 546 -> 588 us with 160).
+template <int L, int F, int S, bool SF, int ILP>
+static __global__ void __launch_bounds__(256) k_union_filter(const uint2* __restrict__ E, uint64_t m, UFState s,
+                                                             CooPart part) {
+    pdl_entry();
+    __shared__ uint2 q[8][64];
+    __shared__ uint32_t qid[8][SF ? 64 : 1];
+    const unsigned lane = lane_id(), warp = threadIdx.x / 32, lt = (1u << lane) - 1;
+    const uint64_t chunks = (m + 31) / 32;
+    const uint64_t sampled = part.mode == COO_ALL ? 0 : (chunks + part.every - 1) / part.every;
+    const uint64_t take = part.mode == COO_SAMPLE ? sampled : chunks - sampled;
+    const uint64_t nw = (uint64_t)gridDim.x * (blockDim.x / 32);
+    unsigned cnt = 0;
+    auto drain = [&](unsigned k) {      // the last k (<= 32) queued unions
+        cnt -= k;
+        if (lane < k) {
+            const uint2 f = q[warp][cnt + lane];
+            Spin sp(s.cap);
+            uf_union<L, F, S, SF>(s, f.x, f.y, SF ? qid[warp][cnt + lane] : 0u, sp);
+        }
+        __syncwarp();
+    };
+    for (uint64_t j0 = ((uint64_t)blockIdx.x * (blockDim.x / 32) + warp) * ILP; j0 < take; j0 += nw * ILP) {
+        if (err_abort(s.err)) return;
+        uint2 e[ILP];
+        uint32_t a[ILP], b[ILP];
+        auto edge_of = [&](int k) -> uint64_t {   // this lane's edge in the k-th chunk
+            const uint64_t j = j0 + k;
+            return (part.mode == COO_SAMPLE ? j * part.every
+                    : part.mode == COO_REST ? j + j / (part.every - 1) + 1 : j) * 32 + lane;
+        };
+#pragma unroll
+        for (int k = 0; k < ILP; ++k) {
+            const uint64_t i = edge_of(k);
+            e[k] = j0 + k < take && i < m ? __ldcs(E + i) : make_uint2(0, 0);
+        }
+#pragma unroll
+        for (int k = 0; k < ILP; ++k) {
+            if (e[k].x >= s.n || e[k].y >= s.n) {
+                atomicOr(s.err, GC_DERR_RANGE);
+                e[k] = make_uint2(0, 0);
+            }
+            a[k] = ldq<true>(s.P, e[k].x);
+            b[k] = ldq<true>(s.P, e[k].y);
+        }
+#pragma unroll
+        for (int k = 0; k < ILP; ++k) {
+            const bool open = a[k] != b[k];
+            const unsigned mk = __ballot_sync(0xFFFFFFFFu, open);
+            if (!mk) continue;
+            if (open) {
+                const unsigned p = cnt + __popc(mk & lt);
+                q[warp][p] = e[k];
+                if (SF) qid[warp][p] = (uint32_t)edge_of(k);
+            }
+            cnt += __popc(mk);
+            __syncwarp();
+            if (cnt >= 32) drain(32);
+        }
+    }
+    if (cnt) drain(cnt);
 }
 
 // k-out sampling (Algorithm 2, first k edges of every vertex).  A warp takes
