@@ -380,6 +380,7 @@ static gconn_status static_run(uint32_t n, uint64_t m, const uint32_t* edges, co
     L2Window l2win;
     l2win.apply(st, P, sizeof(uint32_t) * (size_t)n);
     bool finalized = false;
+    if (!csr && !want_forest && !is_rounds_link(v.link)) GC_TRY(small_cc(v, s, d_edges, m, st, &finalized));
     if (!csr && !finalized) GC_TRY(init_state(s, st));   // csr_connect initialises P and its counters
     if (csr && want_forest)
         GC_TRY(launch("check_arcs", k_check_arcs<OffT>, 1, 1, 0, st, d_off, n, s.err));
