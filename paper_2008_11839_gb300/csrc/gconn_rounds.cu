@@ -9,9 +9,19 @@
 // anything records its number in a control word, and every block reads that
 // word after the round's last barrier to decide, identically, whether to run
 // another round.  No host round trip per round, so these finishes can also be
-// captured into a CUDA graph.  Arrays that other blocks wrote earlier in the
-// same launch are read through L2 (ld.global.cg): L1 is not coherent
-// between blocks.
+// captured into a CUDA graph.  A grid barrier acquires at device scope, so what
+// a phase does not write may be read through L1 in it; what other blocks write
+// in the same phase is read through L2 (ld.global.cg), except where an older
+// value serves as well (said at the place).
+//
+// What bounded the rounds: every edge's message was an atomic, and most aim at a
+// few roots; RMAT n = 2^20, m = 2^24 on one GB300, SV / Liu-Tarjan PRF:
+// 1,292 / 5,260 us at first; no atomic for a message that cannot win, finished
+// edges left out of later rounds (for_live_edges) 605 / 1,034; what a block has
+// sent already remembered in shared memory (SentTable), labels read through L1
+// 375 / 696; compression walks through L1 350 / 629.  1024 x 1024 grid + 16
+// paths of 65,536 (13 to 17 rounds): 864 / 1,064 -> 372 / 482 us, almost all of it the
+// walks through L1.  Blocks per SM: 4, 5, 6, 8 within 2 % but 8 spills (LT 700).
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -63,13 +73,17 @@ __device__ __forceinline__ uint64_t edge_count(uint64_t m_host, const unsigned l
     return m < m_host ? m : m_host;
 }
 
-// FullShortcut while nothing links: every vertex points at its root (a walk
-// through L2), and prev (optional) receives the same value.
+// FullShortcut while nothing links: every vertex points at its root, and prev
+// (optional) receives the same value.  The walk may read through L1: the grid
+// barrier before this phase dropped what L1 held, roots rest, and an entry read
+// before another thread shortened it is an older ancestor on the same path.
+// One walk a thread: two or four in lock step wait for the longest (4 M-vertex
+// grid + paths: 756, 802, 917 us of SV).
 __device__ __forceinline__ void compress_copy(uint32_t n, uint32_t* P, uint32_t* prev, uint32_t* err) {
     for (uint64_t v = gtid(); v < n; v += gstride()) {
         uint32_t p = __ldcg(P + v), r = p;
         for (uint32_t i = 0;; ++i) {
-            uint32_t q = __ldcg(P + r);
+            uint32_t q = __ldca(P + r);
             if (q == r) break;
             r = q;
             if (i == n) { atomicOr(err, GC_DERR_NONCONV); break; }
@@ -90,6 +104,99 @@ __device__ __forceinline__ void finish_rounds(RoundCtl* ctl, uint32_t r) {
     if (gtid() == 0) ctl->rounds = r;
 }
 
+// ------------------------------------------------------------- edge passes
+// The edges of one round, ROUND_ILP chunks of 32 a warp at a time, and the edges
+// that are done left out.  body(i, e) gets arrays of ROUND_ILP edges (an edge
+// that is not taken reads as (0, 0)) and sets keep[k] where edge k can still
+// matter in a later round.
+//
+// live (one bit per edge, a word per chunk) remembers that: round 0 takes every
+// edge and writes the words, later rounds read a word before the edge, so a
+// chunk with no live edge costs a quarter sector instead of 8 of edges and 64 of
+// labels.  A warp meets the same chunks in every round, so only it touches their
+// words.  Null: every edge in every round.
+constexpr int ROUND_ILP = 2;
+
+template <class Body>
+__device__ __forceinline__ void for_live_edges(const uint2* __restrict__ E, uint64_t m, uint32_t n, uint32_t* live,
+                                               uint32_t r, uint32_t* err, Body&& body) {
+    const unsigned lane = lane_id();
+    const uint64_t chunks = (m + 31) / 32, nw = gstride() / 32;
+    for (uint64_t c0 = gtid() / 32 * ROUND_ILP; c0 < chunks; c0 += nw * ROUND_ILP) {
+        uint32_t w[ROUND_ILP], any = 0;
+#pragma unroll
+        for (int k = 0; k < ROUND_ILP; ++k) {
+            w[k] = c0 + k >= chunks ? 0u : live && r ? live[c0 + k] : 0xFFFFFFFFu;
+            any |= w[k];
+        }
+        if (!any) continue;
+        uint2 e[ROUND_ILP];
+        bool keep[ROUND_ILP];
+#pragma unroll
+        for (int k = 0; k < ROUND_ILP; ++k) {
+            const uint64_t i = (c0 + k) * 32 + lane;
+            e[k] = (w[k] >> lane & 1u) && i < m ? __ldcs(E + i) : make_uint2(0, 0);
+        }
+#pragma unroll
+        for (int k = 0; k < ROUND_ILP; ++k)
+            if (e[k].x >= n || e[k].y >= n) {
+                atomicOr(err, GC_DERR_RANGE);
+                e[k] = make_uint2(0, 0);
+            }
+        body(c0 * 32 + lane, e, keep);
+        if (live)
+#pragma unroll
+            for (int k = 0; k < ROUND_ILP; ++k) {
+                const uint32_t x = __ballot_sync(0xFFFFFFFFu, keep[k]);
+                if (lane == 0 && c0 + k < chunks && (x != w[k] || r == 0)) live[c0 + k] = x;
+            }
+    }
+}
+
+// Every vertex that holds a message, which is taken from it; four loads in flight.
+constexpr int MSG_ILP = 4;
+template <class Body>
+__device__ __forceinline__ void for_messages(uint32_t n, unsigned long long* msg, Body&& body) {
+    for (uint64_t x0 = gtid(); x0 < n; x0 += gstride() * MSG_ILP) {
+        unsigned long long mv[MSG_ILP];
+#pragma unroll
+        for (int j = 0; j < MSG_ILP; ++j) mv[j] = x0 + j * gstride() < n ? __ldcg(msg + x0 + j * gstride()) : NOMSG;
+#pragma unroll
+        for (int j = 0; j < MSG_ILP; ++j) {
+            if (mv[j] == NOMSG) continue;
+            msg[x0 + j * gstride()] = NOMSG;
+            body(x0 + j * gstride(), mv[j]);
+        }
+    }
+}
+
+// What this block last sent to a receiver in the current round, one 64-bit word
+// (receiver, value) per slot of a direct-mapped table in shared memory.  Once
+// trees have grown, most edges of a round aim at a few roots; without this every
+// one of them reads the same few L2 sectors, which serve about one request a
+// clock.  A slot that another warp overwrites only costs a repeated message.
+constexpr uint32_t SENT_SLOTS = 512;
+// Fewer edges than this cannot crowd a receiver for long: they send at once, and
+// the reads that spare an atomic would only lengthen the phase (n = 1,000,
+// m = 3,000: SV 34.6 us without, 37.2 with them).
+constexpr uint64_t SENT_MIN_EDGES = 1u << 16;
+struct SentTable {
+    unsigned long long w[SENT_SLOTS];
+    __device__ __forceinline__ void clear() {   // the whole block, at the start of a round
+        for (uint32_t i = threadIdx.x; i < SENT_SLOTS; i += blockDim.x) w[i] = NOMSG;
+        __syncthreads();
+    }
+    // True when this block has sent `to` a value below val, or (ties) val itself.
+    __device__ __forceinline__ bool covered(uint32_t to, uint32_t val, bool ties) const {
+        const unsigned long long x = *(volatile const unsigned long long*)&w[to & (SENT_SLOTS - 1)];
+        const uint32_t v = (uint32_t)x;
+        return (uint32_t)(x >> 32) == to && (v < val || (ties && v == val));
+    }
+    __device__ __forceinline__ void note(uint32_t to, uint32_t val) {
+        *(volatile unsigned long long*)&w[to & (SENT_SLOTS - 1)] = ((unsigned long long)to << 32) | val;
+    }
+};
+
 // --------------------------------------------------------------------- SV
 // Shiloach-Vishkin (Algorithm 12), root-based.  Per round: the hook pass --
 // for each edge the larger of its two current labels is writeMin'ed with the
@@ -98,49 +205,59 @@ __device__ __forceinline__ void finish_rounds(RoundCtl* ctl, uint32_t r) {
 // vertex pass -- then full compression, which also copies the labels into
 // prev.  Stop after a round that hooked nothing.
 template <bool SF>
-__global__ void __launch_bounds__(RB) k_sv(const uint2* __restrict__ E, const uint32_t* eids, uint64_t m_host,
+__global__ void __launch_bounds__(RB, 6) k_sv(const uint2* __restrict__ E, const uint32_t* eids, uint64_t m_host,
                                            const unsigned long long* m_dev, uint32_t n, uint32_t* P, uint32_t* prev,
-                                           unsigned long long* msg, uint32_t* sf, uint32_t* err, RoundCtl* ctl) {
+                                           unsigned long long* msg, uint32_t* sf, uint32_t* live, uint32_t* err,
+                                           RoundCtl* ctl) {
     const uint64_t m = edge_count(m_host, m_dev);
     compress_copy(n, P, prev, err);
     if (SF)
         for (uint64_t x = gtid(); x < n; x += gstride()) msg[x] = NOMSG;
+    __shared__ SentTable sent;
+    const bool crowded = m >= SENT_MIN_EDGES;
     if (!grid_sync(&ctl->bar, err)) return;
     for (uint32_t r = 0;; ++r) {
         if (over_cap(r, err)) return;
         bool ch = false;
-        for (uint64_t i = gtid(); i < m; i += gstride()) {
-            uint2 e = E[i];
-            if (e.x >= n || e.y >= n) { atomicOr(err, GC_DERR_RANGE); continue; }
-            if (SF) {
-                uint32_t pu = __ldcg(prev + e.x), pv = __ldcg(prev + e.y);
-                if (pu == pv) continue;
-                uint32_t lo = min(pu, pv), hi = max(pu, pv);
-                uint32_t id = eids ? eids[i] : (uint32_t)i;
-                atomicMin(msg + hi, ((unsigned long long)lo << 32) | id);
-            } else {
-                uint32_t pu = __ldcg(P + e.x), pv = __ldcg(P + e.y);
-                uint32_t lo = min(pu, pv), hi = max(pu, pv);
-                if (lo != hi && __ldcg(prev + hi) == hi) {
-                    atomicMin(P + hi, lo);
+        if (crowded) sent.clear();
+        for_live_edges(E, m, n, live, r, err, [&](uint64_t i0, uint2 (&e)[ROUND_ILP], bool (&keep)[ROUND_ILP]) {
+            uint32_t lo[ROUND_ILP], hi[ROUND_ILP];
+#pragma unroll
+            for (int k = 0; k < ROUND_ILP; ++k) {
+                // prev is not written in this phase, and a label of P that L1
+                // holds from earlier in it is a label of the same tree
+                const uint32_t* L = SF ? prev : P;
+                const uint32_t pu = __ldca(L + e[k].x), pv = __ldca(L + e[k].y);
+                lo[k] = min(pu, pv);
+                hi[k] = max(pu, pv);
+            }
+#pragma unroll
+            for (int k = 0; k < ROUND_ILP; ++k) {
+                keep[k] = lo[k] != hi[k];   // one tree stays one tree
+                if (!keep[k] || (crowded && sent.covered(hi[k], lo[k], !SF))) continue;
+                if (crowded) sent.note(hi[k], lo[k]);
+                if (SF) {
+                    const uint64_t i = i0 + 32 * k;
+                    const unsigned long long mv = ((unsigned long long)lo[k] << 32) | (eids ? eids[i] : (uint32_t)i);
+                    if (!crowded || __ldcg(msg + hi[k]) > mv) atomicMin(msg + hi[k], mv);
+                } else if ((!crowded || __ldcg(P + hi[k]) > lo[k]) && __ldcg(prev + hi[k]) == hi[k]) {
+                    // (whoever lowered P[hi] this round to lo or below marked the change)
+                    atomicMin(P + hi[k], lo[k]);
                     ch = true;
                 }
             }
-        }
+        });
         if (!SF) mark_changed(ch, &ctl->chg, r);
         if (!grid_sync(&ctl->bar, err)) return;
         if (SF) {   // apply the winning messages to round-start roots
-            for (uint64_t x = gtid(); x < n; x += gstride()) {
-                unsigned long long mv = __ldcg(msg + x);
-                if (mv == NOMSG) continue;
-                msg[x] = NOMSG;
+            for_messages(n, msg, [&](uint64_t x, unsigned long long mv) {
                 uint32_t val = (uint32_t)(mv >> 32);
                 if (__ldcg(P + x) == (uint32_t)x && val < (uint32_t)x) {
                     __stcg(P + x, val);
                     sf[x] = (uint32_t)mv;
                     ch = true;
                 }
-            }
+            });
             mark_changed(ch, &ctl->chg, r);
             if (!grid_sync(&ctl->bar, err)) return;
         }
@@ -164,54 +281,81 @@ __global__ void __launch_bounds__(RB) k_sv(const uint2* __restrict__ E, const ui
 // Shortcut jump per vertex or FullShortcut, then Alter (edge <- (P[u], P[v]),
 // dropped when the ends meet).  Stop after a round that changes neither a
 // parent nor an edge; then full compression.
-__global__ void __launch_bounds__(RB) k_lt(const uint2* __restrict__ E_in, uint2* Ew, const uint32_t* eids,
+__global__ void __launch_bounds__(RB, 6) k_lt(const uint2* __restrict__ E_in, uint2* Ew, const uint32_t* eids,
                                            uint64_t m_host, const unsigned long long* m_dev, uint32_t n, uint32_t* P,
-                                           unsigned long long* msg, uint32_t* sf, int conn, int root_only, int full,
-                                           uint32_t* err, RoundCtl* ctl) {
+                                           unsigned long long* msg, uint32_t* sf, uint32_t* live, int conn,
+                                           int root_only, int full, uint32_t* err, RoundCtl* ctl) {
     const uint64_t m = edge_count(m_host, m_dev);
     const bool alter = Ew != nullptr;
+    __shared__ SentTable sent;
+    const bool crowded = m >= SENT_MIN_EDGES;
     for (uint64_t x = gtid(); x < n; x += gstride()) msg[x] = NOMSG;
     if (!grid_sync(&ctl->bar, err)) return;
     for (uint32_t r = 0;; ++r) {
         if (over_cap(r, err)) return;
         bool ch = false;
-        for (uint64_t i = gtid(); i < m; i += gstride()) {      // Connect
-            uint2 e = alter ? __ldcg(Ew + i) : E_in[i];
-            if (e.x == GC_DINF) continue;                       // dropped by Alter
-            if (e.x >= n || e.y >= n) { atomicOr(err, GC_DERR_RANGE); continue; }
-            if (e.x == e.y) continue;
-            unsigned long long id = eids ? eids[i] : (uint32_t)i;
-            if (conn == GCONN_LT_CONNECT) {
-                atomicMin(msg + e.x, ((unsigned long long)e.y << 32) | id);
-                atomicMin(msg + e.y, ((unsigned long long)e.x << 32) | id);
-            } else {
-                uint32_t pu = __ldcg(P + e.x), pv = __ldcg(P + e.y);
-                if (pu == pv) continue;
-                if (conn == GCONN_LT_PARENT) {
-                    atomicMin(msg + pu, ((unsigned long long)pv << 32) | id);
-                    atomicMin(msg + pv, ((unsigned long long)pu << 32) | id);
+        // Connect.  Every parent is at or below its vertex, so a message that is
+        // not below its receiver is never applied, and one that is not below what
+        // the receiver already holds changes nothing: neither needs the atomic.
+        if (crowded) sent.clear();
+        auto send = [&](uint32_t to, uint32_t val, unsigned long long id) {
+            if (val >= to || (crowded && sent.covered(to, val, !sf))) return;   // (a forest keeps the smallest edge id)
+            if (crowded) sent.note(to, val);
+            const unsigned long long mv = ((unsigned long long)val << 32) | id;
+            if (!crowded || __ldcg(msg + to) > mv) atomicMin(msg + to, mv);
+        };
+        if (conn == GCONN_LT_PARENT && !alter) {
+            for_live_edges(E_in, m, n, live, r, err, [&](uint64_t i0, uint2 (&e)[ROUND_ILP], bool (&keep)[ROUND_ILP]) {
+                uint32_t lo[ROUND_ILP], hi[ROUND_ILP];
+#pragma unroll
+                for (int k = 0; k < ROUND_ILP; ++k) {
+                    const uint32_t pu = __ldca(P + e[k].x), pv = __ldca(P + e[k].y);   // P rests here
+                    lo[k] = min(pu, pv);
+                    hi[k] = max(pu, pv);
+                }
+#pragma unroll
+                for (int k = 0; k < ROUND_ILP; ++k) {
+                    keep[k] = lo[k] != hi[k];
+                    const uint64_t i = i0 + 32 * k;
+                    if (keep[k]) send(hi[k], lo[k], eids ? eids[i] : (uint32_t)i);
+                }
+            });
+        } else {
+            for (uint64_t i = gtid(); i < m; i += gstride()) {
+                uint2 e = alter ? __ldcg(Ew + i) : E_in[i];
+                if (e.x == GC_DINF) continue;                   // dropped by Alter
+                if (e.x >= n || e.y >= n) { atomicOr(err, GC_DERR_RANGE); continue; }
+                if (e.x == e.y) continue;
+                const unsigned long long id = eids ? eids[i] : (uint32_t)i;
+                if (conn == GCONN_LT_CONNECT) {
+                    send(e.x, e.y, id);
+                    send(e.y, e.x, id);
                 } else {
-                    unsigned long long lo = ((unsigned long long)min(pu, pv) << 32) | id;
-                    atomicMin(msg + e.x, lo);
-                    atomicMin(msg + e.y, lo);
-                    atomicMin(msg + pu, lo);
-                    atomicMin(msg + pv, lo);
+                    uint32_t pu = __ldcg(P + e.x), pv = __ldcg(P + e.y);
+                    if (pu == pv) continue;
+                    if (conn == GCONN_LT_PARENT) {
+                        send(pu, pv, id);
+                        send(pv, pu, id);
+                    } else {
+                        const uint32_t lo = min(pu, pv);
+                        send(e.x, lo, id);
+                        send(e.y, lo, id);
+                        send(pu, lo, id);
+                        send(pv, lo, id);
+                    }
                 }
             }
         }
         if (!grid_sync(&ctl->bar, err)) return;
-        for (uint64_t x = gtid(); x < n; x += gstride()) {      // Update / RootUpdate
-            unsigned long long mv = __ldcg(msg + x);
-            if (mv == NOMSG) continue;
-            msg[x] = NOMSG;
+        for_messages(n, msg, [&](uint64_t x, unsigned long long mv) {   // Update / RootUpdate
             uint32_t p = __ldcg(P + x), val = (uint32_t)(mv >> 32);
-            if (root_only && p != (uint32_t)x) continue;
+            if (root_only && p != (uint32_t)x) return;
             if (val < p) {
                 __stcg(P + x, val);
                 if (sf) sf[x] = (uint32_t)mv;
                 ch = true;
             }
-        }
+        });
         mark_changed(ch, &ctl->chg, r);
         if (!grid_sync(&ctl->bar, err)) return;
         ch = false;
@@ -301,8 +445,8 @@ __global__ void __launch_bounds__(RB) k_stergiou(const uint2* __restrict__ E, ui
             if (e.x >= n || e.y >= n) { atomicOr(err, GC_DERR_RANGE); continue; }
             uint32_t a = __ldcg(prev + e.x), b = __ldcg(prev + e.y);
             if (a == b) continue;
-            if (b < a) atomicMin(P + a, b);
-            else atomicMin(P + b, a);
+            const uint32_t lo = min(a, b), hi = max(a, b);
+            if (m < SENT_MIN_EDGES || __ldcg(P + hi) > lo) atomicMin(P + hi, lo);
         }
         if (!grid_sync(&ctl->bar, err)) return;
         bool ch = false;
@@ -411,6 +555,14 @@ struct RoundLaunch {
     }
 };
 
+// One bit per edge for for_live_edges.  Only a saving: a list that the GPU reads
+// in one go does without, and without the memory for it (m / 8 bytes) every
+// round reads every edge.
+static uint32_t* live_bits(DevBuf& buf, uint64_t m, cudaStream_t st) {
+    if (m < SENT_MIN_EDGES || buf.alloc(sizeof(uint32_t) * ((m + 31) / 32), st) != GCONN_OK) return nullptr;
+    return buf.as<uint32_t>();
+}
+
 template <class K>
 unsigned round_grid(K kernel, uint64_t m, uint32_t n) {
     return grid_for(kernel, RB, std::max<uint64_t>(m, n));
@@ -429,9 +581,12 @@ static gconn_status run_sv(const UFState& s, const uint2* E, const uint32_t* eid
     }
     RoundLaunch rl;
     GC_TRY(rl.init(st));
+    DevBuf liveb;
+    // (a caller that counts edge inspections is told of every round's whole pass)
+    uint32_t* live = rounds ? nullptr : live_bits(liveb, m, st);
     auto k = sf ? k_sv<true> : k_sv<false>;
     GC_TRY(launch_coop("sv", k, round_grid(k, m, n), RB, 0, st, E, eids, m, m_dev, n, s.P, prevb.as<uint32_t>(), msg,
-                       s.sf, s.err, rl.ctl));
+                       s.sf, live, s.err, rl.ctl));
     return rounds ? rl.rounds(st, rounds) : GCONN_OK;
 }
 
@@ -452,8 +607,13 @@ static gconn_status run_lt(const Variant& v, const UFState& s, const uint2* E_in
     }
     RoundLaunch rl;
     GC_TRY(rl.init(st));
+    // With ParentConnect and FullShortcut two vertices that share a parent share
+    // it for good (parents are roots, and members follow their root), so their
+    // edge is done.  Other rules can part them again.
+    DevBuf liveb;
+    uint32_t* live = conn == GCONN_LT_PARENT && full && !alter && !rounds ? live_bits(liveb, m, st) : nullptr;
     GC_TRY(launch_coop("lt", k_lt, round_grid(k_lt, m, n), RB, 0, st, E_in, Ew, eids, m, m_dev, n, s.P,
-                       msgb.as<unsigned long long>(), s.sf, conn, (int)root_only, (int)full, s.err, rl.ctl));
+                       msgb.as<unsigned long long>(), s.sf, live, conn, (int)root_only, (int)full, s.err, rl.ctl));
     if (!rounds) return GCONN_OK;
     GC_TRY(rl.rounds(st, rounds));
     *rounds *= (m ? 1u : 0u) + (alter && m ? 1u : 0u);   // connect (+ alter) read every edge
