@@ -221,12 +221,25 @@ def ptr(x):
     raise TypeError(f"cannot take a pointer of {type(x)}")
 
 
+_torch = None    # the torch module, from the first call on
+
+
 def stream_handle(stream=None):
+    """The raw handle of `stream`; None is torch's current stream (the default
+    stream before torch has used the GPU).  A small batch costs the device about
+    2 us and this lookup is made on every call, so the raw handle is read without
+    building a Stream object where torch allows it."""
+    global _torch
     if stream is None:
         try:
-            import torch
-            if torch.cuda.is_available() and torch.cuda.is_initialized():
-                return torch.cuda.current_stream().cuda_stream or None
+            if _torch is None:
+                import torch
+                _torch = torch
+            if _torch.cuda.is_initialized():
+                raw = getattr(_torch._C, "_cuda_getCurrentRawStream", None)
+                if raw is None:
+                    return _torch.cuda.current_stream().cuda_stream or None
+                return raw(_torch.cuda.current_device()) or None
         except Exception:
             pass
         return None
