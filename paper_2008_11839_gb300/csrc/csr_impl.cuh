@@ -258,7 +258,16 @@ gconn_status csr_connect(const Variant& v, const UFState& s, const OffT* off, co
     int L, F, S;
     uf_triple(v, &L, &F, &S);
     int B = block_of(v);
-    GC_TRY(dispatch_uf(L, F, S, s.sf != nullptr, [&]<int l, int f, int sp, bool w>() {
+    GC_TRY(dispatch_uf(L, F, S, s.sf != nullptr, [&]<int l, int f, int sp, bool w>() -> gconn_status {
+        if constexpr (l != LK_JTB) {   // (Union-JTB keeps no parents in P)
+            if (!sampled && n >= (1u << 18)) {
+                auto ka = k_finish_all<l, f, sp, w, OffT>;
+                return launch_pdl("finish", ka, grid_for(ka, B, (uint64_t)n * 32), B, 0, st, off, cols, s,
+                                  (const uint32_t*)small, (const uint32_t*)(cnt + 0), (const unsigned long long*)tasks,
+                                  (const uint32_t*)(cnt + 1), (uint32_t)task_cap, (const uint32_t*)over,
+                                  (const uint32_t*)(cnt + 2));
+            }
+        }
         auto k = k_finish<l, f, sp, w, OffT>;
         return launch_pdl("finish", k, grid_for(k, B, (uint64_t)n * 32), B, 0, st, off, cols, s,
                       (const uint32_t*)active, (const uint32_t*)small, (const uint32_t*)(cnt + 0),

@@ -89,6 +89,53 @@ static __global__ void __launch_bounds__(256) k_union_coo(const uint2* __restric
     }
 }
 
+// A warp's queue of edges whose unions are still to run, in shared memory: push
+// packs the lanes' open edges, and 32 of them run with full lanes as soon as
+// there are 32 (a union takes as long as its longest climb; a warp with a few
+// open edges among closed ones would wait for it with most lanes idle).  Every
+// lane calls every method.  64 entries: at most 31 left over and one row of 32.
+constexpr int QUEUE_WARPS = 8;        // warps of a 256-thread block
+constexpr int QUEUE_LEN = 64;
+template <bool SF>
+struct QueueSmem {
+    uint2 e[QUEUE_WARPS][QUEUE_LEN];
+    uint32_t id[QUEUE_WARPS][SF ? QUEUE_LEN : 1];
+};
+template <int L, int F, int S, bool SF>
+struct UnionQueue {
+    const UFState& s;
+    uint2* e;
+    uint32_t* id;
+    unsigned cnt;
+    __device__ __forceinline__ UnionQueue(const UFState& st, QueueSmem<SF>& m)
+        : s(st), e(m.e[threadIdx.x / 32]), id(m.id[threadIdx.x / 32]), cnt(0) {}
+    __device__ __forceinline__ void drain(unsigned k) {      // the last k (<= 32) entries
+        cnt -= k;
+        if (lane_id() < k) {
+            const uint2 f = e[cnt + lane_id()];
+            Spin sp(s.cap);
+            uf_union<L, F, S, SF>(s, f.x, f.y, SF ? id[cnt + lane_id()] : 0u, sp);
+        }
+        __syncwarp();
+    }
+    template <class Id>
+    __device__ __forceinline__ void push(bool open, uint32_t u, uint32_t v, Id&& edge_id) {
+        const unsigned mk = __ballot_sync(0xFFFFFFFFu, open);
+        if (!mk) return;
+        if (open) {
+            const unsigned p = cnt + __popc(mk & ((1u << lane_id()) - 1));
+            e[p] = make_uint2(u, v);
+            if (SF) id[p] = edge_id();
+        }
+        cnt += __popc(mk);
+        __syncwarp();
+        if (cnt >= 32) drain(32);
+    }
+    __device__ __forceinline__ void finish() {
+        if (cnt) drain(cnt);
+    }
+};
+
 // Which edges a union pass over a COO list takes, in chunks of 32 edges:
 // every chunk, one chunk in `every` (spread over the whole list, so that an
 // ordered list is sampled evenly too), or the chunks that pass left out.
@@ -118,23 +165,13 @@ template <int L, int F, int S, bool SF, int ILP>
 static __global__ void __launch_bounds__(256) k_union_filter(const uint2* __restrict__ E, uint64_t m, UFState s,
                                                              CooPart part) {
     pdl_entry();
-    __shared__ uint2 q[8][64];
-    __shared__ uint32_t qid[8][SF ? 64 : 1];
-    const unsigned lane = lane_id(), warp = threadIdx.x / 32, lt = (1u << lane) - 1;
+    __shared__ QueueSmem<SF> qm;
+    UnionQueue<L, F, S, SF> q(s, qm);
+    const unsigned lane = lane_id(), warp = threadIdx.x / 32;
     const uint64_t chunks = (m + 31) / 32;
     const uint64_t sampled = part.mode == COO_ALL ? 0 : (chunks + part.every - 1) / part.every;
     const uint64_t take = part.mode == COO_SAMPLE ? sampled : chunks - sampled;
     const uint64_t nw = (uint64_t)gridDim.x * (blockDim.x / 32);
-    unsigned cnt = 0;
-    auto drain = [&](unsigned k) {      // the last k (<= 32) queued unions
-        cnt -= k;
-        if (lane < k) {
-            const uint2 f = q[warp][cnt + lane];
-            Spin sp(s.cap);
-            uf_union<L, F, S, SF>(s, f.x, f.y, SF ? qid[warp][cnt + lane] : 0u, sp);
-        }
-        __syncwarp();
-    };
     for (uint64_t j0 = ((uint64_t)blockIdx.x * (blockDim.x / 32) + warp) * ILP; j0 < take; j0 += nw * ILP) {
         if (err_abort(s.err)) return;
         uint2 e[ILP];
@@ -159,21 +196,10 @@ static __global__ void __launch_bounds__(256) k_union_filter(const uint2* __rest
             b[k] = ldq<true>(s.P, e[k].y);
         }
 #pragma unroll
-        for (int k = 0; k < ILP; ++k) {
-            const bool open = a[k] != b[k];
-            const unsigned mk = __ballot_sync(0xFFFFFFFFu, open);
-            if (!mk) continue;
-            if (open) {
-                const unsigned p = cnt + __popc(mk & lt);
-                q[warp][p] = e[k];
-                if (SF) qid[warp][p] = (uint32_t)edge_of(k);
-            }
-            cnt += __popc(mk);
-            __syncwarp();
-            if (cnt >= 32) drain(32);
-        }
+        for (int k = 0; k < ILP; ++k)
+            q.push(a[k] != b[k], e[k].x, e[k].y, [&] { return (uint32_t)edge_of(k); });
     }
-    if (cnt) drain(cnt);
+    q.finish();
 }
 
 // k-out sampling (Algorithm 2, first k edges of every vertex).  A warp takes
@@ -977,6 +1003,115 @@ __global__ void __launch_bounds__(256) k_finish(const OffT* __restrict__ off, co
     uint32_t ct = *ntasks;
     if (ct > task_cap) ct = task_cap;
     finish_pass<L, F, S, SF, OffT, false>(off, cols, s, active, small, *nsmall, tasks, ct, over, *nover);
+}
+
+// The finish of an unsampled pass (every vertex with an arc is listed, each edge
+// is taken from its larger endpoint, and most edges of a dense graph join
+// nothing): the columns of a whole task and the parents of its smaller
+// neighbours are in flight together, the unequal ones queued (as k_union_filter;
+// one gather an edge, the row's own parent is read once).  A list of at least 16
+// vertices a warp is compared and queued too.  RMAT without sampling: n = 2^20,
+// m = 2^24 266 -> 188 us a pass, Union-Async 960 -> 558; n = 2^22, m = 2^26
+// 831 -> 528 (716 with 40 registers a thread, which spill).  Below 2^18 vertices
+// the unions contend and comparing first only delays them (ER n = 16,384,
+// m = 65,536: 60 -> 66 us): k_finish.  After sampling nearly every listed arc joins two trees and the
+// lists are short: k_finish (there the compared parents and the extra registers
+// cost 53 -> 67 us on grid + paths of 8.4 M vertices).
+template <int L, int F, int S, bool SF, class OffT = uint64_t>
+__global__ void __launch_bounds__(256, 5) k_finish_all(const OffT* __restrict__ off, const uint32_t* __restrict__ cols,
+                                                    UFState s, const uint32_t* small, const uint32_t* nsmall,
+                                                    const unsigned long long* tasks, const uint32_t* ntasks,
+                                                    uint32_t task_cap, const uint32_t* over, const uint32_t* nover) {
+    pdl_entry();
+    __shared__ QueueSmem<SF> qm;
+    UnionQueue<L, F, S, SF> q(s, qm);
+    uint32_t ct = *ntasks;
+    if (ct > task_cap) ct = task_cap;
+    const uint32_t cs = *nsmall, co = *nover;
+    const uint64_t nw = (uint64_t)gridDim.x * (blockDim.x / 32);
+    const uint64_t gw = (uint64_t)blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32;
+    const unsigned lane = lane_id();
+    // one row of at most ROWS * 32 arcs [lo, hi) of vertex u
+    constexpr int ROWS = TASK_ARCS / 32;
+    auto row = [&](uint32_t u, uint64_t lo, uint64_t hi) {
+        const uint32_t pu = ldq<true>(s.P, u);
+        uint32_t v[ROWS], pv[ROWS];
+#pragma unroll
+        for (int k = 0; k < ROWS; ++k) {
+            const uint64_t a = lo + 32 * k + lane;
+            v[k] = a < hi ? cols[a] : u;
+        }
+#pragma unroll
+        for (int k = 0; k < ROWS; ++k) {
+            if (v[k] >= s.n) {
+                atomicOr(s.err, GC_DERR_RANGE);
+                v[k] = u;
+            }
+            pv[k] = v[k] < u ? ldq<true>(s.P, v[k]) : pu;
+        }
+#pragma unroll
+        for (int k = 0; k < ROWS; ++k)
+            q.push(pv[k] != pu, u, v[k], [&] { return (uint32_t)(lo + 32 * k + lane); });
+    };
+    for (uint64_t t = gw; t < ct; t += nw) {
+        if (err_abort(s.err)) return;
+        const unsigned long long task = tasks[t];
+        const uint32_t u = (uint32_t)(task >> 32);
+        row(u, (uint64_t)off[u] + (task & 0xFFFFFFFFull) * TASK_ARCS, off[u + 1]);
+    }
+    q.finish();
+    // low-degree vertices, flattened per warp as in finish_pass
+    uint64_t G = ((uint64_t)cs + nw - 1) / nw;
+    G = G < 1 ? 1 : G > 32 ? 32 : G;
+    const bool queued = G >= 16;
+    for (uint64_t base = gw * G; base < cs; base += nw * G) {
+        if (err_abort(s.err)) return;
+        const uint64_t i = base + lane;
+        uint32_t u = 0, d = 0;
+        uint64_t lo = 0;
+        if (lane < G && i < cs) {
+            u = small[i];
+            lo = off[u];
+            d = (uint32_t)(off[u + 1] - lo);
+        }
+        uint32_t inc = d;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            uint32_t t = __shfl_up_sync(0xFFFFFFFFu, inc, o);
+            if ((int)lane >= o) inc += t;
+        }
+        const uint32_t total = __shfl_sync(0xFFFFFFFFu, inc, 31), exc = inc - d;
+        for (uint32_t jb = 0; jb < total; jb += 32) {
+            const uint32_t j = jb + lane;
+            int l0 = 0, l1 = 31;                       // first lane whose inclusive sum exceeds j
+#pragma unroll
+            for (int step = 0; step < 5; ++step) {
+                int mid = (l0 + l1) >> 1;
+                uint32_t vm = __shfl_sync(0xFFFFFFFFu, inc, mid);
+                if (vm > j) l1 = mid; else l0 = mid + 1;
+            }
+            const uint32_t ou = __shfl_sync(0xFFFFFFFFu, u, l0);
+            const uint64_t a = __shfl_sync(0xFFFFFFFFu, lo, l0) + (j - __shfl_sync(0xFFFFFFFFu, exc, l0));
+            uint32_t v = j < total ? cols[a] : ou;
+            if (v >= s.n) {
+                atomicOr(s.err, GC_DERR_RANGE);
+                v = ou;
+            }
+            if (queued) {
+                q.push(v < ou && ldq<true>(s.P, ou) != ldq<true>(s.P, v), ou, v, [&] { return (uint32_t)a; });
+            } else if (v < ou) {
+                Spin sp(s.cap);
+                uf_union<L, F, S, SF>(s, ou, v, (uint32_t)a, sp);
+            }
+        }
+    }
+    q.finish();
+    for (uint64_t i = gw; i < co; i += nw) {
+        const uint32_t u = over[i];
+        const uint64_t hi = off[u + 1];
+        for (uint64_t lo = off[u]; lo < hi; lo += TASK_ARCS) row(u, lo, hi);
+    }
+    q.finish();
 }
 
 // Finish without vertex gathering (measurement form, GCONN_ABL_NO_VG): one
