@@ -101,7 +101,7 @@ gconn_status union_coo_static(const Variant& v, const UFState& s, const uint32_t
             const bool dense = m >= 4 * n;   // most edges join nothing
             // rules that compress nothing on the way (naive finds of
             // Union-Async and Union-Hooks, Afforest)
-            constexpr bool bare = f == FD_NAIVE && (l == LK_ASYNC || l == LK_HOOKS || l == LK_AFFOREST);
+            constexpr bool bare = rule_is_bare<l, f>();
             if (bare && n < (1u << 15)) return union_coo(v, s, edges, m, 0, st);
             if (n >= (1u << 15) && (bare || n <= (1u << 19)) && m >= 2 * n) {
                 const uint32_t every = (uint32_t)std::min<uint64_t>(4 * m / (3 * n), 1u << 30);

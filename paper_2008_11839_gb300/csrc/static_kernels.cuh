@@ -225,6 +225,17 @@ struct KoutJob {
 // compression happened) and re-run later from its endpoints by
 // k_union_jobs, so a few long climbs do not hold 31 idle lanes.
 constexpr uint32_t KOUT_FAST_STEPS = 8;
+// HB's second step under rules that compress nothing on the way (naive finds),
+// from HB_LONG_N vertices: there the walks are long whoever runs them, and a
+// deferred union only starts again.  RMAT n = 10^6, Union-Async: 8 steps 110 us a
+// pass, 16 97, 20 95, 32 97; ER n = 2^20 224 -> 200.  Fewer vertices contend and
+// gain from deferral (ER n = 65,536: 60 -> 65), and so do the rules that compress
+// (Union-Rem-CAS on ER n = 2^20: 85 -> 100) and k-out (RMAT n = 2^22: no gain, ER
+// n = 2^20: 81 -> 98).
+// The budget is a template argument: as a run-time value it costs the default
+// rule 17 % (the unrolled climb).
+constexpr uint32_t HB_LONG_STEPS = 16;
+constexpr uint32_t HB_LONG_N = 1u << 19;
 
 struct JobQueue {
     KoutJob* jobs;
@@ -234,11 +245,11 @@ struct JobQueue {
 
 // One union under the soft budget when a queue is given: an abandoned union
 // goes to the queue (or, if it is full, runs on with the full cap).
-template <int L, int F, int S, bool SF>
+template <int L, int F, int S, bool SF, uint32_t STEPS = KOUT_FAST_STEPS>
 __device__ __forceinline__ void union_or_defer(const UFState& s, const JobQueue& dq, uint32_t a, uint32_t b,
                                                uint32_t eid) {
     if (dq.jobs) {
-        Spin fast(KOUT_FAST_STEPS, true);
+        Spin fast(STEPS, true);
         uf_union<L, F, S, SF>(s, a, b, eid, fast);
         if (!fast.dead) return;
         unsigned long long slot = atomicAdd(dq.count, 1ull);
@@ -515,7 +526,7 @@ static __global__ void k_hb_init(const OffT* __restrict__ off, const uint32_t* _
 // would leave most lanes idle while a few run four unions in sequence.
 constexpr int HB_WARP_N = 4;
 
-template <int L, int F, int S, bool SF, class OffT = uint64_t>
+template <int L, int F, int S, bool SF, class OffT = uint64_t, uint32_t STEPS = KOUT_FAST_STEPS>
 static __global__ void __launch_bounds__(256) k_hb2w(const OffT* __restrict__ off,
                                                      const uint32_t* __restrict__ cols, int N, UFState s,
                                                      JobQueue dq) {
@@ -564,7 +575,7 @@ static __global__ void __launch_bounds__(256) k_hb2w(const OffT* __restrict__ of
         __syncwarp();
         for (unsigned j = lane; j < total; j += 32) {
             KoutJob jb = my[j];
-            union_or_defer<L, F, S, SF>(s, dq, jb.u, jb.v, jb.eid);
+            union_or_defer<L, F, S, SF, STEPS>(s, dq, jb.u, jb.v, jb.eid);
         }
         __syncwarp();
         lo0 = lo1; hi0 = hi1;

@@ -487,6 +487,12 @@ __device__ __forceinline__ bool same_root_lockstep(const UFState& s, uint32_t x,
     return true;
 }
 
+// Rules that compress nothing on the way.
+template <int L, int F>
+__host__ __device__ constexpr bool rule_is_bare() {
+    return F == FD_NAIVE && (L == LK_ASYNC || L == LK_HOOKS || L == LK_AFFOREST);
+}
+
 // ----------------------------------------------------------- dispatcher
 template <int L, int F, int S, bool SF>
 __device__ __forceinline__ bool uf_union(const UFState& s, uint32_t u, uint32_t v, uint32_t eid, Spin& sp) {
