@@ -105,7 +105,8 @@ static gconn_status launch_class(gconn_batch* b, int c, int block, int rule, cud
     const size_t smem = smem_cc_bytes(b->cls_maxn[c], block);
     int per_sm = 0;
     void* kf = smem_kernel(rule, wide);
-    GC_CUDA(cudaFuncSetAttribute(kf, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    // always the largest block's size: plans made by several threads share the attribute
+    GC_CUDA(cudaFuncSetAttribute(kf, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BLOCK_MAX));
     GC_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kf, block, smem));
     if (per_sm < 1) return GCONN_E_UNSUPPORTED;
     uint32_t grid = (uint32_t)std::min<uint64_t>((uint64_t)per_sm * num_sms(), cnt);

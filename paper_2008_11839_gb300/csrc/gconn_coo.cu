@@ -46,7 +46,8 @@ gconn_status small_cc(const Variant& v, const UFState& s, const uint32_t* edges,
            : rule == BR_ASYNC_NAIVE ? k_small_cc<BR_ASYNC_NAIVE> : k_small_cc<BR_ASYNC_HALVE>;
     const int B = 1024;
     const size_t smem = smem_cc_bytes(s.n, B);
-    GC_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    // always the form's largest size: calls from several threads share the attribute
+    GC_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_cc_bytes(SMALL_CC_N, B)));
     *done = true;
     return launch_pdl("small_cc", k, 1, B, smem, st, s.n, (const uint2*)edges, (uint32_t)m, s.P, s.err);
 }

@@ -196,9 +196,10 @@ __device__ __forceinline__ void smem_cc(uint32_t* smem, uint32_t n, const uint2*
 
 // Shared memory of one block for graphs of up to max_n vertices, and whether
 // 32-bit parents fit beside the queues and the static words.
+constexpr int SMEM_BLOCK_MAX = 227 * 1024 - 64;   // beside the kernels' static words
 inline size_t smem_queue_bytes(int block) { return sizeof(uint32_t) * BATCH_QUEUE * (size_t)(block / 32); }
 inline bool smem_wide(uint32_t max_n, int block) {
-    return 4ull * max_n + smem_queue_bytes(block) + 64 <= 227ull * 1024;
+    return 4ull * max_n + smem_queue_bytes(block) <= (uint64_t)SMEM_BLOCK_MAX;
 }
 inline size_t smem_cc_bytes(uint32_t max_n, int block) {
     return smem_queue_bytes(block) + (smem_wide(max_n, block) ? sizeof(uint32_t) * (size_t)max_n
