@@ -28,12 +28,26 @@ namespace gc {
 
 constexpr int NCLS = GCONN_BATCH_CLASSES;
 constexpr uint32_t SMEM_MAX_N = 65536;
+// The form of a class's kernel, by its edges per thread of a block (mean over the
+// class).  Eight rows of edges at a time cost 64 registers a thread, so half the
+// blocks of a small class are resident: from 64 edges a thread the loads in
+// flight are worth it.  Below, two rows a turn (31 registers), and below 4 edges a
+// thread its own unions without the queue (24).  Microseconds a batch, one union
+// per thread / eight rows / two rows / direct: 8,192 graphs of 128 to 1,024
+// vertices, m = n 55 / 80 / 59 / 53 (2.2 edges a thread), m = 4n 95 / 109 / 86 / 95
+// (9); 65,536 graphs of 8 to 32 vertices 124 / 286 / 154 / 127; 4,096 graphs of 1,000
+// to 4,096, m = 12n 268 / 268 / 265 / 367 (120); 300 graphs of 16,384 to 50,000, m = 4n
+// 207 / 159 / 178 / 275 (518).  Blocks of one warp lose no resident block to the
+// registers and keep eight rows (m = 16n on 32 to 128 vertices, 40 edges a thread:
+// 66 / 49 / 68).
+constexpr uint64_t BATCH_FULL = 64, BATCH_LEAN = 4;
+
 // Persistent class kernel: CTAs pull graph indices (largest first) from an
 // atomic queue; each graph: init parents in shared memory, stream its edges,
 // union, then write every vertex's root (its min-id label) to global memory
 // (smem_cc).
-template <int R, class T>
-__global__ void __launch_bounds__(1024, 1) k_batch_smem(const uint64_t* __restrict__ vo, const uint64_t* __restrict__ eo,
+template <int R, class T, int ILP>
+__global__ void __launch_bounds__(1024, ILP < BATCH_ILP ? 2 : 1) k_batch_smem(const uint64_t* __restrict__ vo, const uint64_t* __restrict__ eo,
                              const uint2* __restrict__ E, uint32_t* __restrict__ labels,
                              const uint32_t* __restrict__ order, uint32_t count, uint32_t* queue, uint32_t* err) {
     extern __shared__ uint32_t smem_raw[];
@@ -47,7 +61,7 @@ __global__ void __launch_bounds__(1024, 1) k_batch_smem(const uint64_t* __restri
         uint64_t vb = vo[g];
         uint32_t n = (uint32_t)(vo[g + 1] - vb);
         uint64_t eb = eo[g], m = eo[g + 1] - eb;
-        smem_cc<R, T>(smem_raw, n, E + eb, m, labels + vb, err);
+        smem_cc<R, T, ILP>(smem_raw, n, E + eb, m, labels + vb, err);
     }
 }
 
@@ -70,6 +84,7 @@ struct gconn_batch {
     uint32_t* queues = nullptr;     // one counter per class
     uint32_t cls_begin[NCLS + 1];
     uint32_t cls_maxn[NCLS];
+    uint64_t cls_edges[NCLS];       // edges of the class's graphs together
     std::vector<uint32_t> large;    // graphs above the last class
     std::vector<uint64_t> hvo, heo;
     cudaStream_t side[NCLS] = {};
@@ -86,15 +101,12 @@ static int rule_of(int link, int find) {
     return find == GCONN_FIND_HALVE ? BR_ASYNC_HALVE : BR_ASYNC_NAIVE;
 }
 
-static void* smem_kernel(int rule, bool wide) {
-    if (wide) {
-        if (rule == BR_REM_SPLIT) return (void*)k_batch_smem<BR_REM_SPLIT, uint32_t>;
-        if (rule == BR_ASYNC_HALVE) return (void*)k_batch_smem<BR_ASYNC_HALVE, uint32_t>;
-        return (void*)k_batch_smem<BR_ASYNC_NAIVE, uint32_t>;
-    }
-    if (rule == BR_REM_SPLIT) return (void*)k_batch_smem<BR_REM_SPLIT, uint16_t>;
-    if (rule == BR_ASYNC_HALVE) return (void*)k_batch_smem<BR_ASYNC_HALVE, uint16_t>;
-    return (void*)k_batch_smem<BR_ASYNC_NAIVE, uint16_t>;
+using BatchKernel = void (*)(const uint64_t*, const uint64_t*, const uint2*, uint32_t*, const uint32_t*, uint32_t,
+                             uint32_t*, uint32_t*);
+template <class T, int ILP>
+static BatchKernel rule_kernel(int rule) {
+    return rule == BR_REM_SPLIT ? k_batch_smem<BR_REM_SPLIT, T, ILP>
+         : rule == BR_ASYNC_HALVE ? k_batch_smem<BR_ASYNC_HALVE, T, ILP> : k_batch_smem<BR_ASYNC_NAIVE, T, ILP>;
 }
 
 // Launch one class's persistent kernel on stream st.
@@ -103,28 +115,18 @@ static gconn_status launch_class(gconn_batch* b, int c, int block, int rule, cud
     if (!cnt) return GCONN_OK;
     const bool wide = smem_wide(b->cls_maxn[c], block);   // 32-bit parents (no 16-bit CAS)
     const size_t smem = smem_cc_bytes(b->cls_maxn[c], block);
+    const uint64_t threads = (uint64_t)block * cnt, m = b->cls_edges[c];
+    const BatchKernel k = !wide ? rule_kernel<uint16_t, BATCH_ILP>(rule)
+                        : block == 32 || m >= BATCH_FULL * threads ? rule_kernel<uint32_t, BATCH_ILP>(rule)
+                        : m >= BATCH_LEAN * threads ? rule_kernel<uint32_t, 2>(rule) : rule_kernel<uint32_t, 1>(rule);
     int per_sm = 0;
-    void* kf = smem_kernel(rule, wide);
     // always the largest block's size: plans made by several threads share the attribute
-    GC_CUDA(cudaFuncSetAttribute(kf, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BLOCK_MAX));
-    GC_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kf, block, smem));
+    GC_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BLOCK_MAX));
+    GC_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, block, smem));
     if (per_sm < 1) return GCONN_E_UNSUPPORTED;
     uint32_t grid = (uint32_t)std::min<uint64_t>((uint64_t)per_sm * num_sms(), cnt);
-    const uint32_t* ord = b->order + b->cls_begin[c];
-    uint32_t* q = b->queues + c;
-    uint32_t* err = err_word();
-    const uint2* E = (const uint2*)b->edges;
-#define GC_BLAUNCH(RR, TT) \
-    return launch("batch_smem", k_batch_smem<RR, TT>, grid, block, smem, st, b->vo, b->eo, E, b->labels, ord, cnt, q, err)
-    if (wide) {
-        if (rule == BR_REM_SPLIT) GC_BLAUNCH(BR_REM_SPLIT, uint32_t);
-        if (rule == BR_ASYNC_HALVE) GC_BLAUNCH(BR_ASYNC_HALVE, uint32_t);
-        GC_BLAUNCH(BR_ASYNC_NAIVE, uint32_t);
-    }
-    if (rule == BR_REM_SPLIT) GC_BLAUNCH(BR_REM_SPLIT, uint16_t);
-    if (rule == BR_ASYNC_HALVE) GC_BLAUNCH(BR_ASYNC_HALVE, uint16_t);
-    GC_BLAUNCH(BR_ASYNC_NAIVE, uint16_t);
-#undef GC_BLAUNCH
+    return launch("batch_smem", k, grid, block, smem, st, b->vo, b->eo, (const uint2*)b->edges, b->labels,
+                  b->order + b->cls_begin[c], cnt, b->queues + c, err_word());
 }
 
 // The whole batch on `st`: reset queues, fork one stream per class, join,
@@ -261,8 +263,13 @@ static gconn_status batch_build(uint32_t G, const uint64_t* vtx_off, const uint6
         });
         b->cls_begin[c] = (uint32_t)order.size();
         uint32_t mx = 0;
-        for (uint32_t g : cls[c]) mx = std::max<uint32_t>(mx, (uint32_t)(b->hvo[g + 1] - b->hvo[g]));
+        uint64_t edges_c = 0;
+        for (uint32_t g : cls[c]) {
+            mx = std::max<uint32_t>(mx, (uint32_t)(b->hvo[g + 1] - b->hvo[g]));
+            edges_c += b->heo[g + 1] - b->heo[g];
+        }
         b->cls_maxn[c] = mx;
+        b->cls_edges[c] = edges_c;
         order.insert(order.end(), cls[c].begin(), cls[c].end());
     }
     b->cls_begin[NCLS] = (uint32_t)order.size();

@@ -13,7 +13,7 @@ namespace gc {
 constexpr uint32_t SMEM_CAP = 1u << 20;   // loop cap per shared-memory union
 
 enum { BR_ASYNC_NAIVE = 0, BR_ASYNC_HALVE = 1, BR_REM_SPLIT = 2 };
-constexpr int BATCH_ILP = 8;    // rows of 32 edges a warp checks at a time
+constexpr int BATCH_ILP = 8;    // most rows of 32 edges a warp checks at a time
 constexpr int BATCH_ROWS = 4;   // ... and queues before it drains
 constexpr int BATCH_QUEUE = 32 + 32 * BATCH_ROWS;   // queued unions per warp (at most 31 left over)
 
@@ -87,6 +87,33 @@ __device__ __forceinline__ void sm_union_async(volatile T* P, uint32_t u, uint32
     if (!left) atomicOr(err, GC_DERR_NONCONV);
 }
 
+// One whole union of a thread.
+template <int R, class T>
+__device__ __forceinline__ void sm_union(volatile T* P, uint32_t u, uint32_t v, uint32_t* err) {
+    if constexpr (R == BR_REM_SPLIT) {
+        for (uint32_t left = SMEM_CAP; left; --left)
+            if (sm_rem_step<T>(P, u, v)) return;
+        atomicOr(err, GC_DERR_NONCONV);
+    } else {
+        sm_union_async<R, T>(P, u, v, err);
+    }
+}
+
+// Every vertex's root to global memory; all threads of the block, after their unions.
+template <class T>
+__device__ __forceinline__ void sm_labels(volatile T* P, uint32_t n, uint32_t* __restrict__ labels) {
+    for (uint32_t i = threadIdx.x; i < n; i += blockDim.x) {
+        uint32_t r = i, left = SMEM_CAP;
+        while (left--) {
+            uint32_t p = sm_ld(P, r);
+            if (p == r) break;
+            r = p;
+        }
+        labels[i] = r;
+    }
+    __syncthreads();
+}
+
 // A large graph's edges mostly join nothing (a mean degree of 4 to 32 against
 // one link per vertex), and a union of 32 edges in lock step takes as many
 // steps as its longest climb.  So a warp first compares the parents of
@@ -106,6 +133,10 @@ __device__ __forceinline__ void sm_union_async(volatile T* P, uint32_t u, uint32
 // 918; draining after each row instead of every four 997 (the drain is inlined
 // once per place, and registers bound the co-resident classes).
 //
+// ILP rows of 32 edges a turn of a warp; 1: a union per thread, no queue.  The
+// block's rows follow one another (row k of a turn lies blockDim edges after row
+// k - 1), so that a list shorter than a turn still gives every warp its share.
+//
 // Every thread of the block calls; smem holds smem_cc_bytes() bytes.
 template <int R, class T, int ILP = BATCH_ILP>
 __device__ __forceinline__ void smem_cc(uint32_t* smem, uint32_t n, const uint2* __restrict__ E, uint64_t m,
@@ -116,6 +147,16 @@ __device__ __forceinline__ void smem_cc(uint32_t* smem, uint32_t n, const uint2*
     volatile T* P = reinterpret_cast<volatile T*>(smem + (blockDim.x / 32) * BATCH_QUEUE);
     for (uint32_t i = threadIdx.x; i < n; i += blockDim.x) P[i] = (T)i;
     __syncthreads();
+    if constexpr (ILP == 1) {   // a union per thread, no queue
+        for (uint64_t j = threadIdx.x; j < m; j += blockDim.x) {
+            const uint2 e = __ldcs(E + j);
+            if (e.x >= n || e.y >= n) atomicOr(err, GC_DERR_RANGE);
+            else if (e.x != e.y) sm_union<R, T>(P, e.x, e.y, err);
+        }
+        __syncthreads();
+        sm_labels(P, n, labels);
+        return;
+    }
     unsigned cnt = 0;        // the warp's queued unions
     auto drain = [&](unsigned take) {   // one turn of the last `take` (<= 32) queued pairs
         cnt -= take;
@@ -133,7 +174,8 @@ __device__ __forceinline__ void smem_cc(uint32_t* smem, uint32_t n, const uint2*
         cnt += __popc(mk);
         __syncwarp();
     };
-    auto check = [&](uint2 (&e)[ILP]) {
+    // `rows` (the same in the whole warp) of the ILP rows hold edges
+    auto check = [&](uint2 (&e)[ILP], int rows) {
         uint32_t top = 0;
 #pragma unroll
         for (int k = 0; k < ILP; ++k) top = max(top, max(e[k].x, e[k].y));
@@ -146,13 +188,16 @@ __device__ __forceinline__ void smem_cc(uint32_t* smem, uint32_t n, const uint2*
         uint32_t a[ILP], b[ILP];
 #pragma unroll
         for (int k = 0; k < ILP; ++k) {
+            if (k >= rows) break;
             a[k] = sm_ld(P, e[k].x);
             b[k] = sm_ld(P, e[k].y);
         }
 #pragma unroll
         for (int h = 0; h < ILP; h += ROWS) {
+            if (h >= rows) break;
 #pragma unroll
             for (int k = h; k < h + ROWS; ++k) {
+                if (k >= rows) break;
                 const bool open = a[k] != b[k];
                 const unsigned mk = __ballot_sync(0xFFFFFFFFu, open);
                 if (open) uq[cnt + __popc(mk & lt)] = e[k].x | (e[k].y << 16);
@@ -163,35 +208,27 @@ __device__ __forceinline__ void smem_cc(uint32_t* smem, uint32_t n, const uint2*
         }
     };
     constexpr uint64_t PIECE = 1u << 30;   // edges per 32-bit index range
+    const uint32_t B = blockDim.x;
     for (uint64_t m0 = 0; m0 < m; m0 += PIECE) {
         const uint32_t len = (uint32_t)(m - m0 < PIECE ? m - m0 : PIECE);
-        const uint2* Eg = E + m0 + lane;
-        uint32_t j = warp * 32 * ILP;
+        const uint2* Eg = E + m0 + threadIdx.x;
+        uint32_t j = 0;
         uint2 e[ILP];
-        for (; j + 32 * ILP <= len; j += blockDim.x * ILP) {
+        for (; j + B * ILP <= len; j += B * ILP) {
 #pragma unroll
-            for (int k = 0; k < ILP; ++k) e[k] = __ldcs(Eg + j + k * 32);
-            check(e);
+            for (int k = 0; k < ILP; ++k) e[k] = __ldcs(Eg + j + k * B);
+            check(e, ILP);
         }
-        if (j < len) {
+        if (j + warp * 32 < len) {   // the last turn: the rows that are left, spread over the warps
 #pragma unroll
             for (int k = 0; k < ILP; ++k)
-                e[k] = j + k * 32 + lane < len ? __ldcs(Eg + j + k * 32) : make_uint2(0, 0);
-            check(e);
+                e[k] = j + k * B + threadIdx.x < len ? __ldcs(Eg + j + k * B) : make_uint2(0, 0);
+            check(e, (int)((len - j - warp * 32 + B - 1) / B));
         }
     }
     while (cnt) drain(min(cnt, 32u));
     __syncthreads();
-    for (uint32_t i = threadIdx.x; i < n; i += blockDim.x) {
-        uint32_t r = i, left = SMEM_CAP;
-        while (left--) {
-            uint32_t p = sm_ld(P, r);
-            if (p == r) break;
-            r = p;
-        }
-        labels[i] = r;
-    }
-    __syncthreads();
+    sm_labels(P, n, labels);
 }
 
 // Shared memory of one block for graphs of up to max_n vertices, and whether
