@@ -133,9 +133,8 @@ __device__ __forceinline__ void sm_labels(volatile T* P, uint32_t n, uint32_t* _
 // 918; draining after each row instead of every four 997 (the drain is inlined
 // once per place, and registers bound the co-resident classes).
 //
-// ILP rows of 32 edges a turn of a warp; 1: a union per thread, no queue.  The
-// block's rows follow one another (row k of a turn lies blockDim edges after row
-// k - 1), so that a list shorter than a turn still gives every warp its share.
+// ILP rows of 32 edges a turn of a warp; 1: a union per thread, no queue.  What is
+// left of a list below a turn of the block is spread over its warps row by row.
 //
 // Every thread of the block calls; smem holds smem_cc_bytes() bytes.
 template <int R, class T, int ILP = BATCH_ILP>
@@ -174,8 +173,7 @@ __device__ __forceinline__ void smem_cc(uint32_t* smem, uint32_t n, const uint2*
         cnt += __popc(mk);
         __syncwarp();
     };
-    // `rows` (the same in the whole warp) of the ILP rows hold edges
-    auto check = [&](uint2 (&e)[ILP], int rows) {
+    auto check = [&](uint2 (&e)[ILP]) {
         uint32_t top = 0;
 #pragma unroll
         for (int k = 0; k < ILP; ++k) top = max(top, max(e[k].x, e[k].y));
@@ -188,16 +186,13 @@ __device__ __forceinline__ void smem_cc(uint32_t* smem, uint32_t n, const uint2*
         uint32_t a[ILP], b[ILP];
 #pragma unroll
         for (int k = 0; k < ILP; ++k) {
-            if (k >= rows) break;
             a[k] = sm_ld(P, e[k].x);
             b[k] = sm_ld(P, e[k].y);
         }
 #pragma unroll
         for (int h = 0; h < ILP; h += ROWS) {
-            if (h >= rows) break;
 #pragma unroll
             for (int k = h; k < h + ROWS; ++k) {
-                if (k >= rows) break;
                 const bool open = a[k] != b[k];
                 const unsigned mk = __ballot_sync(0xFFFFFFFFu, open);
                 if (open) uq[cnt + __popc(mk & lt)] = e[k].x | (e[k].y << 16);
@@ -210,20 +205,20 @@ __device__ __forceinline__ void smem_cc(uint32_t* smem, uint32_t n, const uint2*
     constexpr uint64_t PIECE = 1u << 30;   // edges per 32-bit index range
     const uint32_t B = blockDim.x;
     for (uint64_t m0 = 0; m0 < m; m0 += PIECE) {
-        const uint32_t len = (uint32_t)(m - m0 < PIECE ? m - m0 : PIECE);
-        const uint2* Eg = E + m0 + threadIdx.x;
-        uint32_t j = 0;
+        const uint32_t len = (uint32_t)(m - m0 < PIECE ? m - m0 : PIECE), full = len - len % (B * ILP);
+        const uint2* Eg = E + m0 + lane;
         uint2 e[ILP];
-        for (; j + B * ILP <= len; j += B * ILP) {
+        for (uint32_t j = warp * 32 * ILP; j < full; j += B * ILP) {
 #pragma unroll
-            for (int k = 0; k < ILP; ++k) e[k] = __ldcs(Eg + j + k * B);
-            check(e, ILP);
+            for (int k = 0; k < ILP; ++k) e[k] = __ldcs(Eg + j + k * 32);
+            check(e);
         }
-        if (j + warp * 32 < len) {   // the last turn: the rows that are left, spread over the warps
+        const uint32_t j = full + warp * 32;
+        if (j < len) {   // less than a turn of the block
 #pragma unroll
             for (int k = 0; k < ILP; ++k)
-                e[k] = j + k * B + threadIdx.x < len ? __ldcs(Eg + j + k * B) : make_uint2(0, 0);
-            check(e, (int)((len - j - warp * 32 + B - 1) / B));
+                e[k] = j + k * B + lane < len ? __ldcs(Eg + j + k * B) : make_uint2(0, 0);
+            check(e);
         }
     }
     while (cnt) drain(min(cnt, 32u));
