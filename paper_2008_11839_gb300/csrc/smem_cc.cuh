@@ -10,7 +10,13 @@
 
 namespace gc {
 
-constexpr uint32_t SMEM_CAP = 1u << 20;   // loop cap per shared-memory union
+constexpr uint32_t SMEM_CAP = 1u << 20;   // loop cap of a thread's own union
+// Cap of the turns that empty a warp's queue.  A queued pair's climb takes fewer
+// than 2^18 turns: a turn lowers one of two ids below 2^16 or loses the one
+// compare-and-swap that a root can lose.  So 160 pairs, at 32 a turn, are done in
+// 5 x 2^18 turns; beyond the cap an invariant is broken.  (No measurable cost:
+// 4,096 graphs 918-920 us without, 917-920 with it.)
+constexpr uint32_t SMEM_TURNS = 1u << 21;
 
 enum { BR_ASYNC_NAIVE = 0, BR_ASYNC_HALVE = 1, BR_REM_SPLIT = 2 };
 constexpr int BATCH_ILP = 8;    // most rows of 32 edges a warp checks at a time
@@ -173,6 +179,16 @@ __device__ __forceinline__ void smem_cc(uint32_t* smem, uint32_t n, const uint2*
         cnt += __popc(mk);
         __syncwarp();
     };
+    auto drain_below = [&](unsigned low) {   // until fewer than `low` pairs are queued
+        for (uint32_t left = SMEM_TURNS; cnt >= low; --left) {
+            if (!left) {
+                atomicOr(err, GC_DERR_NONCONV);
+                cnt = 0;
+                break;
+            }
+            drain(min(cnt, 32u));
+        }
+    };
     auto check = [&](uint2 (&e)[ILP]) {
         uint32_t top = 0;
 #pragma unroll
@@ -199,7 +215,7 @@ __device__ __forceinline__ void smem_cc(uint32_t* smem, uint32_t n, const uint2*
                 cnt += __popc(mk);
             }
             __syncwarp();
-            while (cnt >= 32) drain(32);
+            drain_below(32);
         }
     };
     constexpr uint64_t PIECE = 1u << 30;   // edges per 32-bit index range
@@ -221,7 +237,7 @@ __device__ __forceinline__ void smem_cc(uint32_t* smem, uint32_t n, const uint2*
             check(e);
         }
     }
-    while (cnt) drain(min(cnt, 32u));
+    drain_below(1);
     __syncthreads();
     sm_labels(P, n, labels);
 }
