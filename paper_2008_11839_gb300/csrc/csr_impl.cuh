@@ -324,11 +324,11 @@ static gconn_status static_run(uint32_t n, uint64_t m, const uint32_t* edges, co
     const uint32_t* d_edges = edges;
     const OffT* d_off = off;
     const uint32_t* d_cols = cols;
-    bool any_host = false;
+    bool any_host = false, edges_host = false;
     if (!csr) {
         if (m) {
-            bool h = !is_device_ptr(edges);
-            any_host |= h;
+            edges_host = !is_device_ptr(edges);
+            any_host |= edges_host;
             // a union-find finish reads every edge once: host edges are read
             // in place where the device can; the round finishes re-read them
             if (is_rounds_link(v.link))
@@ -391,7 +391,8 @@ static gconn_status static_run(uint32_t n, uint64_t m, const uint32_t* edges, co
     L2Window l2win;
     l2win.apply(st, P, sizeof(uint32_t) * (size_t)n);
     bool finalized = false;
-    if (!csr && !want_forest && !is_rounds_link(v.link)) GC_TRY(small_cc(v, s, d_edges, m, st, &finalized));
+    if (!csr && !want_forest && !is_rounds_link(v.link)) 
+        GC_TRY(small_cc(v, s, d_edges, m, edges_host, st, &finalized));
     if (!csr && !finalized) GC_TRY(init_state(s, st));   // csr_connect initialises P and its counters
     if (csr && want_forest)
         GC_TRY(launch("check_arcs", k_check_arcs<OffT>, 1, 1, 0, st, d_off, n, s.err));

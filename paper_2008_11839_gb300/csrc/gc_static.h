@@ -16,8 +16,8 @@ gconn_status init_state(const UFState& s, cudaStream_t st, uint32_t* zero = null
 gconn_status union_coo(const Variant& v, const UFState& s, const uint32_t* edges, uint64_t m, uint32_t eid_base,
                        cudaStream_t st);
 gconn_status union_coo_static(const Variant& v, const UFState& s, const uint32_t* edges, uint64_t m, cudaStream_t st);
-gconn_status small_cc(const Variant& v, const UFState& s, const uint32_t* edges, uint64_t m, cudaStream_t st,
-                      bool* done);
+gconn_status small_cc(const Variant& v, const UFState& s, const uint32_t* edges, uint64_t m, bool host,
+                      cudaStream_t st, bool* done);
 gconn_status compress_all(const Variant& v, const UFState& s, cudaStream_t st);
 gconn_status finalize_labels(const Variant& v, const UFState& s, uint32_t* labels, cudaStream_t st);
 gconn_status sf_output(uint32_t n, const uint32_t* sf, uint64_t* forest, uint64_t* count, cudaStream_t st);

@@ -24,30 +24,48 @@ static __global__ void __launch_bounds__(1024, 1) k_small_cc(uint32_t n, const u
 // The whole static pass of a small COO graph in one block, with the variant's
 // own rule (the three that smem_cc has); *done says whether the call took it.
 // Three dependent kernels cost their launch gaps and L2 round trips whatever
-// the size; one block walks 32 edges a turn per warp in shared memory.  A call
-// on n = 1,000, m = 4,000: 23.4 -> 17.2 us (the host's share of a call); n = 16,000:
-// m = 32,000 34 -> 28 us, m = 64,000 45 -> 34 us, m = 128,000 no gain, so the
-// line lies at 65,536 edges.  A caller's own iteration cap counts the steps of
-// the global-memory rules: those calls keep them.
-constexpr uint32_t SMALL_CC_N = 16384;
-constexpr uint64_t SMALL_CC_M = 65536;
+// the size; one block walks 32 edges a turn per warp in shared memory.  The
+// limits, by rule (microseconds of the kernels in a captured plan, three kernels
+// -> one block):
+// - Rem-CAS climbs one step a turn with full lanes: n = 1,000, m = 4,000 16 -> 8,
+//   m = 64,000 27 -> 18; n = 16,384, m = 32,768 36 -> 30 (ER), 22 -> 18 (RMAT),
+//   m = 65,536 43 -> 36, 33 -> 25; m = 128,000 no gain.
+// - Union-Async runs a whole union per lane, so a turn takes as long as its longest
+//   walk.  Halving keeps the walks short: n = 4,096, m = 4,096 21 -> 13, m = 65,536
+//   37 -> 28; but n = 16,384, m = 32,768 29 -> 41.  Naive walks grow with the
+//   list: n = 1,000, m = 1,000 14 -> 10, m = 4,000 18 -> 20; n = 4,096, m = 16,384
+//   23 -> 53.
+// Host lists are read in place over the host link, by this one SM: wall time a
+// call, page-locked, n = 16,384: Rem-CAS m = 32,768 57 -> 57, m = 65,536 67 -> 71;
+// halving n = 4,096, m = 16,384 43 -> 42, m = 32,768 47 -> 48.
+// A caller's own iteration cap counts the steps of the global-memory rules: those
+// calls keep them.
+struct SmallLimit {
+    uint32_t n, m, m_host;
+};
+static SmallLimit small_limit(int rule) {
+    return rule == BR_REM_SPLIT ? SmallLimit{16384, 65536, 32768}
+         : rule == BR_ASYNC_HALVE ? SmallLimit{4096, 65536, 16384} : SmallLimit{16384, 1024, 1024};
+}
 
-gconn_status small_cc(const Variant& v, const UFState& s, const uint32_t* edges, uint64_t m, cudaStream_t st,
-                      bool* done) {
+gconn_status small_cc(const Variant& v, const UFState& s, const uint32_t* edges, uint64_t m, bool host,
+                      cudaStream_t st, bool* done) {
     *done = false;
-    if (s.n > SMALL_CC_N || m > SMALL_CC_M || v.cap != DEFAULT_CAP) return GCONN_OK;
+    if (v.cap != DEFAULT_CAP) return GCONN_OK;
     int L, F, S;
     uf_triple(v, &L, &F, &S);
     const int rule = L == LK_REMCAS && F == FD_NAIVE && S == SP_SPLIT_ONE ? BR_REM_SPLIT
                    : L == LK_ASYNC && F == FD_NAIVE ? BR_ASYNC_NAIVE
                    : L == LK_ASYNC && F == FD_HALVE ? BR_ASYNC_HALVE : -1;
     if (rule < 0) return GCONN_OK;
+    const SmallLimit lim = small_limit(rule);
+    if (s.n > lim.n || m > (host ? lim.m_host : lim.m)) return GCONN_OK;
     auto k = rule == BR_REM_SPLIT ? k_small_cc<BR_REM_SPLIT>
            : rule == BR_ASYNC_NAIVE ? k_small_cc<BR_ASYNC_NAIVE> : k_small_cc<BR_ASYNC_HALVE>;
     const int B = 1024;
     const size_t smem = smem_cc_bytes(s.n, B);
-    // always the form's largest size: calls from several threads share the attribute
-    GC_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_cc_bytes(SMALL_CC_N, B)));
+    // always the rule's largest size: calls from several threads share the attribute
+    GC_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_cc_bytes(lim.n, B)));
     *done = true;
     return launch_pdl("small_cc", k, 1, B, smem, st, s.n, (const uint2*)edges, (uint32_t)m, s.P, s.err);
 }

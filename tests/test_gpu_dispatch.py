@@ -1,0 +1,60 @@
+"""Which kernels a call launches: the size, rule and memory lines of the
+dispatch, on both sides of each line, with the results against the oracle."""
+import numpy as np
+import pytest
+
+import graphgen
+import oracle
+import paper_2008_11839_gb300 as g
+from gpu_util import dev, host_u32
+
+pytestmark = pytest.mark.gpu
+
+
+def kernels_of(call):
+    """Names of the kernels that `call` launches."""
+    g.gconn_profile_enable(True)
+    try:
+        g.gconn_profile_sync()
+        g.gconn_profile_reset()
+        call()
+        g.gconn_sync()
+        g.gconn_profile_sync()
+        return {k for k, v in g.gconn_profile_get().items() if v[0]}
+    finally:
+        g.gconn_profile_enable(False)
+
+
+def cc_kernels(n, m, edges, v, ref):
+    import torch
+    lab = torch.empty(n, dtype=torch.int32, device="cuda")
+    names = kernels_of(lambda: g.gconn_cc(n, m, edges, lab, v))
+    assert (host_u32(lab) == ref).all()
+    return names
+
+
+@pytest.mark.parametrize("rule,n,m,one_block", [
+    (("remcas", "naive"), 16384, 65536, True), (("remcas", "naive"), 16384, 65537, False),
+    (("remcas", "naive"), 16385, 20000, False),
+    (("async", "halve"), 4096, 65536, True), (("async", "halve"), 4097, 9000, False),
+    (("async", "naive"), 4096, 1024, True), (("async", "naive"), 4096, 1025, False),
+    (("async", "naive"), 4096, 20000, False), (("async", "naive"), 16384, 1000, True)])
+def test_one_block_limits_on_device_lists(rule, n, m, one_block):
+    g.build()
+    e = graphgen.er(n, m, n + m)
+    v = g.make_variant(link=rule[0], find=rule[1], splice="split_one" if rule[0] == "remcas" else "none")
+    assert ("small_cc" in cc_kernels(n, m, dev(e), v, oracle.cc_uf(n, e))) == one_block
+
+
+@pytest.mark.parametrize("rule,n,m,one_block", [
+    (("remcas", "naive"), 16000, 32768, True), (("remcas", "naive"), 16000, 32769, False),
+    (("async", "halve"), 4000, 16384, True), (("async", "halve"), 4000, 16385, False),
+    (("async", "naive"), 4000, 1024, True), (("async", "naive"), 4000, 1025, False)])
+@pytest.mark.parametrize("pinned", [False, True])
+def test_one_block_limits_on_host_lists(rule, n, m, one_block, pinned):
+    import torch
+    g.build()
+    e = graphgen.er(n, m, n + m)
+    h = torch.from_numpy(e.view(np.int32)).pin_memory() if pinned else e
+    v = g.make_variant(link=rule[0], find=rule[1], splice="split_one" if rule[0] == "remcas" else "none")
+    assert ("small_cc" in cc_kernels(n, m, h, v, oracle.cc_uf(n, e))) == one_block
