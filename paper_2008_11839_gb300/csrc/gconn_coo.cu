@@ -38,8 +38,8 @@ static __global__ void __launch_bounds__(1024, 1) k_small_cc(uint32_t n, const u
 // Host lists are read in place over the host link, by this one SM: wall time a
 // call, page-locked, n = 16,384: Rem-CAS m = 32,768 57 -> 57, m = 65,536 67 -> 71;
 // halving n = 4,096, m = 16,384 43 -> 42, m = 32,768 47 -> 48.
-// A caller's own iteration cap counts the steps of the global-memory rules: those
-// calls keep them.
+// A caller's own iteration cap counts the steps of the global-memory rules, and a
+// caller's own block size is meant for them: those calls keep them.
 struct SmallLimit {
     uint32_t n, m, m_host;
 };
@@ -51,7 +51,7 @@ static SmallLimit small_limit(int rule) {
 gconn_status small_cc(const Variant& v, const UFState& s, const uint32_t* edges, uint64_t m, bool host,
                       cudaStream_t st, bool* done) {
     *done = false;
-    if (v.cap != DEFAULT_CAP) return GCONN_OK;
+    if (v.cap != DEFAULT_CAP || v.block > 0) return GCONN_OK;
     int L, F, S;
     uf_triple(v, &L, &F, &S);
     const int rule = L == LK_REMCAS && F == FD_NAIVE && S == SP_SPLIT_ONE ? BR_REM_SPLIT

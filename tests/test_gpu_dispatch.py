@@ -58,3 +58,13 @@ def test_one_block_limits_on_host_lists(rule, n, m, one_block, pinned):
     h = torch.from_numpy(e.view(np.int32)).pin_memory() if pinned else e
     v = g.make_variant(link=rule[0], find=rule[1], splice="split_one" if rule[0] == "remcas" else "none")
     assert ("small_cc" in cc_kernels(n, m, h, v, oracle.cc_uf(n, e))) == one_block
+
+
+@pytest.mark.parametrize("kw", [dict(block=64), dict(block=256), dict(iter_cap=1 << 20)])
+def test_own_block_size_or_cap_keeps_the_global_memory_kernels(kw):
+    g.build()
+    n, m = 3000, 9000
+    e = graphgen.er(n, m, 1)
+    ref = oracle.cc_uf(n, e)
+    assert "small_cc" in cc_kernels(n, m, dev(e), g.make_variant(link="remcas", splice="split_one"), ref)
+    assert "small_cc" not in cc_kernels(n, m, dev(e), g.make_variant(link="remcas", splice="split_one", **kw), ref)
