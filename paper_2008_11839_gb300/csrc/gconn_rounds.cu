@@ -557,9 +557,13 @@ struct RoundLaunch {
 
 // One bit per edge for for_live_edges.  Only a saving: a list that the GPU reads
 // in one go does without, and without the memory for it (m / 8 bytes) every
-// round reads every edge.
+// round reads every edge.  A captured pass does without too: there the allocation
+// is a node of the plan, and where it does not fit the whole plan fails.
 static uint32_t* live_bits(DevBuf& buf, uint64_t m, cudaStream_t st) {
-    if (m < SENT_MIN_EDGES || buf.alloc(sizeof(uint32_t) * ((m + 31) / 32), st) != GCONN_OK) return nullptr;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (m < SENT_MIN_EDGES || cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone)
+        return nullptr;
+    if (buf.alloc(sizeof(uint32_t) * ((m + 31) / 32), st) != GCONN_OK) return nullptr;
     return buf.as<uint32_t>();
 }
 
