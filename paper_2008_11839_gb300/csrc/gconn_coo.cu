@@ -88,21 +88,38 @@ gconn_status union_coo(const Variant& v, const UFState& s, const uint32_t* edges
     });
 }
 
-// The COO finish of a static pass (every vertex a singleton at the start).
-// Three forms, by size:
-// - fewer edges than fill the GPU once (m < 49,152): one union per thread;
-//   comparing first only adds a round trip (ER n = 16,000, m = 32,000: 34 against
-//   53 us).
-// - 2^15 <= n <= 2^19 and m >= 2n: as many threads as vertices or more would
-//   start on singletons at once and contend for the same few roots.  So about
-//   3n/4 edges, spread over the list, are united first (where a random graph's
-//   giant component appears), the trees are flattened, and the other edges then
-//   mostly find equal parents.  ER n = 65,536, m = 2^20: 98 -> 49 us (85 without
-//   the first pass; a sample of n/2 or n edges 80, 50); n = 200,000, m = 16n:
-//   168 -> 80 (98); RMAT n = 400,000, m = 8n: 144 -> 82 (84).  Above 2^19 the
-//   first wave no longer covers the vertices (RMAT n = 10^6: 156 us without,
-//   173 with); at 16,000 vertices the two launches cost what they save (45, 48).
-// - otherwise one pass over all edges.
+// The COO finish of a static pass (every vertex a singleton at the start) has
+// three forms: a union per thread (k_union_coo), one compared-and-queued pass over
+// all edges (k_union_filter), and a sampled one: about 3n/4 to n edges, spread over
+// the list, are united first (where a random graph's giant component appears),
+// the trees are flattened, and the other edges then mostly find equal parents.
+// Measured at 13 sizes of n from 12,000 to 2^22, m from n/2 to 16n, on ER, RMAT and
+// grid + paths lists, by rule (m / n and microseconds: union per thread, chosen
+// form).  The lines lie where neither kind of graph loses:
+// - Fewer edges than the resident threads of 152 SMs (m < 49,152): comparing first
+//   only adds a round trip (ER n = 32,768, m = n, Rem-CAS: 25 against 32).
+// - 2^15 <= n <= 2^19: as many threads as vertices or more would start on singletons
+//   at once and contend for the same few roots: sampled.  Rem with naive finds
+//   from max(2n, 2^17) edges: ER n = 65,536 x 2 65, 44; x 16 101, 54; RMAT n = 2^18 x 8
+//   139, 66; but n = 46,000 x 2 ER 60, 43 and RMAT 26, 35.  Union-Async with compressing
+//   finds and Union-Hooks from 2n (n = 2^15 x 2: 81, 67; 86, 67).  Rules that shorten
+//   their own walks (Early; split and halve) have less to gain: from max(2n, 2^18)
+//   (Early, ER n = 2^18 x 4 69, 56; n = 92,000 x 2 32, 42), and Early with such a find
+//   not at all (split, ER n = 131,072 x 8 81, 157; RMAT n = 2^18 x 8 167, 112).
+//   Their second pass takes 8 rows of edges from 2^17 vertices and 4n edges (ER
+//   n = 131,072 x 8, Early: 94 with 2 rows, 59 with 8), every other takes 2 (ER n = 2^15
+//   x 4, Rem-CAS: 44; 44 with 2, 54 with 8).  Rules that compress nothing are sampled
+//   at any n from 2^15: from 3n edges, from 2^18 vertices 2n (Union-Async, ER n = 65,536 x 2
+//   63, 62, x 3 83, 63; n = 2^22 x 8 1,476, 503; Afforest, n = 65,536 x 2 30, 37).
+// - n < 2^15: sampled from 8n edges (12,000 x 8: ER 55, 38, RMAT 25, 26), below one
+//   pass (16,384 x 4: ER 55, 47, RMAT 23, 24); rules that shorten their own walks
+//   sampled from 16n, else a union per thread, as are the rules that compress
+//   nothing and Early with a compressing find.
+// - n > 2^19: the first wave no longer covers the vertices; one pass from n edges
+//   (n = 10^6 x 2: ER 182, 100, RMAT 76, 72; 2^22 x 1 257, 186).  Below, nearly every edge
+//   links (n = 2^20 x 1/2: 40, 44; and at n <= 2^19 below 2n: grid + paths of 393,216
+//   81, 104).  Rules that shorten their own walks up to 2^20 only from 4n (n = 10^6,
+//   Early: ER x 8 147, 137, RMAT x 2 58, 77).
 gconn_status union_coo_static(const Variant& v, const UFState& s, const uint32_t* edges, uint64_t m, cudaStream_t st) {
     if (v.link == GCONN_LINK_JTB || m < 49152) return union_coo(v, s, edges, m, 0, st);
     int L, F, S;
@@ -112,23 +129,41 @@ gconn_status union_coo_static(const Variant& v, const UFState& s, const uint32_t
     return dispatch_uf(L, F, S, s.sf != nullptr, [&]<int l, int f, int sp, bool sf>() -> gconn_status {
         if constexpr (l == LK_JTB) return GCONN_E_UNSUPPORTED;   // handled above
         else {
-            auto pass = [&](const char* name, bool dense, CooPart part, uint64_t count) {
-                auto k = dense ? k_union_filter<l, f, sp, sf, 8> : k_union_filter<l, f, sp, sf, 2>;
-                return launch_pdl(name, k, grid_for(k, B, count / (dense ? 8 : 2) + 1), B, 0, st, (const uint2*)edges,
+            auto pass = [&](const char* name, bool wide, CooPart part, uint64_t count) {
+                auto k = wide ? k_union_filter<l, f, sp, sf, 8> : k_union_filter<l, f, sp, sf, 2>;
+                return launch_pdl(name, k, grid_for(k, B, count / (wide ? 8 : 2) + 1), B, 0, st, (const uint2*)edges,
                                   m, s, part);
             };
-            const bool dense = m >= 4 * n;   // most edges join nothing
-            // rules that compress nothing on the way (naive finds of
-            // Union-Async and Union-Hooks, Afforest)
-            constexpr bool bare = rule_is_bare<l, f>();
-            if (bare && n < (1u << 15)) return union_coo(v, s, edges, m, 0, st);
-            if (n >= (1u << 15) && (bare || n <= (1u << 19)) && m >= 2 * n) {
-                const uint32_t every = (uint32_t)std::min<uint64_t>(4 * m / (3 * n), 1u << 30);
+            auto sampled = [&](bool wide) -> gconn_status {
+                const uint32_t every = (uint32_t)std::min<uint64_t>(4 * m / (3 * n), 1u << 30);   // >= 2
                 GC_TRY(pass("union_coo_sample", false, CooPart{COO_SAMPLE, every}, m / every + 32));
                 GC_TRY(finalize_labels(v, s, s.P, st));
-                return pass("union_coo", dense, CooPart{COO_REST, every}, m);
+                return pass("union_coo", wide, CooPart{COO_REST, every}, m);
+            };
+            auto one_pass = [&](bool wide) { return pass("union_coo", wide, CooPart{COO_ALL, 0}, m); };
+            auto per_thread = [&] { return union_coo(v, s, edges, m, 0, st); };
+
+            constexpr bool hooks = l == LK_HOOKS, bare = rule_is_bare<l, f>();
+            constexpr bool shortens = l == LK_EARLY || (!hooks && (f == FD_SPLIT || f == FD_HALVE));
+            constexpr bool early_find = l == LK_EARLY && f != FD_NAIVE;
+            if (n > (1u << 19) && !bare) {
+                if (shortens && n <= (1u << 20)) return m >= 4 * n ? one_pass(true) : per_thread();
+                return m < n ? per_thread() : one_pass(m >= (shortens || l == LK_REMLOCK ? 4 : 2) * n);
             }
-            return pass("union_coo", dense, CooPart{COO_ALL, 0}, m);
+            if (bare && m < 2 * n) {
+                if (hooks ? 2 * m >= 3 * n : l != LK_AFFOREST && n > (1u << 19) && m >= n) return one_pass(false);
+                return per_thread();
+            }
+            if (early_find || (bare && n < (1u << 15))) return per_thread();
+            if (n < (1u << 15)) {
+                if (m >= (shortens ? 16 : 8) * n) return sampled(false);
+                return shortens ? per_thread() : one_pass(false);
+            }
+            const uint64_t least = hooks || (l == LK_ASYNC && f == FD_COMPRESS) ? 2 * n
+                                 : bare ? (n >= (1u << 18) ? 2 : 3) * n
+                                 : std::max<uint64_t>(2 * n, 1u << (shortens ? 18 : 17));
+            if (m < least) return per_thread();
+            return sampled(shortens && n >= (1u << 17) && m >= 4 * n);
         }
     });
 }

@@ -67,9 +67,9 @@ static __global__ void k_init(uint32_t n, uint32_t* P, uint32_t* H, u64w* W, uin
     }
 }
 
-// Insert batches (Section 3.5), and Union-JTB's COO finish: one union per
-// edge, grid-stride, edges streamed once.  eid_base offsets the recorded
-// forest ids.
+// Insert batches (Section 3.5), Union-JTB's COO finish, and the static COO lists
+// that comparing first does not pay for: one union per edge, grid-stride, edges
+// streamed once.  eid_base offsets the recorded forest ids.
 template <int L, int F, int S, bool SF>
 static __global__ void __launch_bounds__(256) k_union_coo(const uint2* __restrict__ E, uint64_t m, UFState s,
                                                    uint32_t eid_base) {
@@ -156,11 +156,12 @@ struct CooPart {
 // a union per thread (k_union_coo), 530 us here, of which the two gathers an
 // edge account for 430 us.  RMAT n = 10^6, m = 1.6 x 10^7: 294 -> 156 us;
 // 4096 x 4096 grid + 64 paths of 2^18 (m = 1.45 n): 2,796 -> 2,182 us.
-// ILP by density: where most edges link (m < 4n) the compared parents are used
-// again by the union, and more edges in flight only push them out of L1 (grid +
-// paths: 2,182, 2,499, 2,803 us with 2, 4, 8); dense lists want the loads in
-// flight (RMAT n = 2^22: 571, 546, 530 us).  A queue of more than 64 entries a
-// warp costs more L1 than it saves (RMAT n = 2^22: 546 -> 588 us with 160).
+// ILP: where most edges link, and after a sampled first pass on small vertex sets,
+// the compared parents are used again by the union, and more edges in flight only
+// push them out of L1 (grid + paths: 2,182, 2,499, 2,803 us with 2, 4, 8); long dense
+// lists want the loads in flight (RMAT n = 2^22: 571, 546, 530 us).  A queue of more
+// than 64 entries a warp costs more L1 than it saves (RMAT n = 2^22: 546 -> 588 us
+// with 160).
 template <int L, int F, int S, bool SF, int ILP>
 static __global__ void __launch_bounds__(256) k_union_filter(const uint2* __restrict__ E, uint64_t m, UFState s,
                                                              CooPart part) {

@@ -68,3 +68,42 @@ def test_own_block_size_or_cap_keeps_the_global_memory_kernels(kw):
     ref = oracle.cc_uf(n, e)
     assert "small_cc" in cc_kernels(n, m, dev(e), g.make_variant(link="remcas", splice="split_one"), ref)
     assert "small_cc" not in cc_kernels(n, m, dev(e), g.make_variant(link="remcas", splice="split_one", **kw), ref)
+
+
+# (rule, n, m, sampled first pass)
+COO_LINES = [
+    ("remcas", "naive", "split_one", 40000, (1 << 17) - 1, False), ("remcas", "naive", "split_one", 40000, 1 << 17, True),
+    ("remcas", "naive", "splice", 70000, 139999, False), ("remcas", "naive", "splice", 70000, 140000, True),
+    ("remcas", "naive", "split_one", 9000, 71999, False), ("remcas", "naive", "split_one", 9000, 72000, True),
+    ("remcas", "naive", "split_one", (1 << 19) + 1, 1 << 21, False),
+    ("remcas", "halve", "halve_one", 40000, (1 << 18) - 1, False), ("remcas", "halve", "halve_one", 40000, 1 << 18, True),
+    ("early", "naive", "none", 140000, 279999, False), ("early", "naive", "none", 140000, 280000, True),
+    ("early", "naive", "none", 140000, 560000, True), ("early", "split", "none", 140000, 560000, False),
+    ("early", "naive", "none", 9000, 143999, False), ("early", "naive", "none", 9000, 144000, True),
+    ("async", "naive", "none", 40000, 119999, False), ("async", "naive", "none", 40000, 120000, True),
+    ("async", "naive", "none", 1 << 18, (1 << 19) - 1, False), ("async", "naive", "none", 1 << 18, 1 << 19, True),
+    ("async", "naive", "none", 600000, 1200000, True), ("async", "naive", "none", 600000, 700000, False),
+    ("async", "compress", "none", 33000, 65999, False), ("async", "compress", "none", 33000, 66000, True),
+    ("async", "naive", "none", 30000, 400000, False), ("hooks", "naive", "none", 33000, 66000, True),
+    ("hooks", "naive", "none", 50000, 80000, False), ("afforest", "naive", "none", 600000, 900000, False),
+    ("early", "naive", "none", 600000, 1300000, False), ("early", "naive", "none", 600000, 2400000, False),
+    ("remlock", "naive", "split_one", 600000, 1300000, False)]
+
+
+@pytest.mark.parametrize("link,find,splice,n,m,sampled", COO_LINES)
+def test_coo_finish_lines(link, find, splice, n, m, sampled):
+    g.build()
+    e = graphgen.er(n, m, n + m)
+    names = cc_kernels(n, m, dev(e), g.make_variant(link=link, find=find, splice=splice), oracle.cc_uf(n, e))
+    assert ("union_coo_sample" in names) == sampled and "union_coo" in names
+
+
+@pytest.mark.parametrize("n,m", [(40000, 70000), (9000, 60000), (9000, 80000), (300000, 450000), (600000, 500000)])
+def test_coo_forests_around_the_lines(n, m):
+    g.build()
+    e = graphgen.er(n, m, n + m)
+    ref = oracle.cc_uf(n, e)
+    for link, find, splice in (("remcas", "naive", "split_one"), ("early", "halve", "none"), ("async", "naive", "none")):
+        ids, _ = g.spanning_forest(n, dev(e), g.make_variant(link=link, find=find, splice=splice))
+        g.gconn_sync()
+        assert oracle.sf_check(n, e, ids.cpu().numpy().astype(np.uint64), ref) == 0
