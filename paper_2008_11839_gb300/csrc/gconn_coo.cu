@@ -118,8 +118,9 @@ gconn_status union_coo(const Variant& v, const UFState& s, const uint32_t* edges
 // - n > 2^19: the first wave no longer covers the vertices; one pass from n edges
 //   (n = 10^6 x 2: ER 182, 100, RMAT 76, 72; 2^22 x 1 257, 186).  Below, nearly every edge
 //   links (n = 2^20 x 1/2: 40, 44; and at n <= 2^19 below 2n: grid + paths of 393,216
-//   81, 104).  Rules that shorten their own walks up to 2^20 only from 4n (n = 10^6,
-//   Early: ER x 8 147, 137, RMAT x 2 58, 77).
+//   81, 104).  Rules that shorten their own walks up to 2^20 only from 8n (Early,
+//   n = 10^6: ER x 8 147, 137, RMAT x 2 58, 77; n = 2^20: ER x 4 106, 121), and
+//   Union-Async not there (split, RMAT n = 2^20 x 16 245, 289).
 gconn_status union_coo_static(const Variant& v, const UFState& s, const uint32_t* edges, uint64_t m, cudaStream_t st) {
     if (v.link == GCONN_LINK_JTB || m < 49152) return union_coo(v, s, edges, m, 0, st);
     int L, F, S;
@@ -147,7 +148,8 @@ gconn_status union_coo_static(const Variant& v, const UFState& s, const uint32_t
             constexpr bool shortens = l == LK_EARLY || (!hooks && (f == FD_SPLIT || f == FD_HALVE));
             constexpr bool early_find = l == LK_EARLY && f != FD_NAIVE;
             if (n > (1u << 19) && !bare) {
-                if (shortens && n <= (1u << 20)) return m >= 4 * n ? one_pass(true) : per_thread();
+                if (shortens && n <= (1u << 20))
+                    return l != LK_ASYNC && m >= 8 * n ? one_pass(true) : per_thread();
                 return m < n ? per_thread() : one_pass(m >= (shortens || l == LK_REMLOCK ? 4 : 2) * n);
             }
             if (bare && m < 2 * n) {
