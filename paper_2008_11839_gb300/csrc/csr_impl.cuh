@@ -260,21 +260,35 @@ gconn_status csr_connect(const Variant& v, const UFState& s, const OffT* off, co
     int L, F, S;
     uf_triple(v, &L, &F, &S);
     int B = block_of(v);
+    // Without sampling the compared-and-queued finish: from 2^20 vertices on any
+    // list (ER, m = n/2 to 16n, RMAT and grids, every rule: 0.34 to 1.1 of the pass
+    // with k_finish), from 2^18 on lists of at least 16 arcs a vertex (Union-Async 8,
+    // Early 32), where fewer edges link (Rem-CAS, ER n = 2^18: m = 2n 94 -> 99 us, 4n
+    // 108 -> 122, 8n 133 -> 128, 16n 195 -> 129; Union-Async n = 2^19: m = n 98 -> 102, 4n
+    // 251 -> 171; Early n = 2^18: 8n 104 -> 113, 16n 162 -> 138).  Below 2^18 the unions
+    // contend and comparing first only delays them (ER n = 2^17, m = 4n, Early:
+    // 71 -> 87).  Where the device makes the choice, the kernel that does not work
+    // costs about 1.3 us of a pass of 33 us and more.
+    const uint64_t never = UINT64_MAX;
+    uint64_t dense = sampled || jtb || n < (1u << 18) ? never
+                   : n >= (1u << 20) ? 0 : (uint64_t)n * (L == LK_ASYNC ? 8 : L == LK_EARLY ? 32 : 16);
+    if (dense && dense != never && csr_arcs_hint() != UINT64_MAX) dense = csr_arcs_hint() >= dense ? 0 : never;
     GC_TRY(dispatch_uf(L, F, S, s.sf != nullptr, [&]<int l, int f, int sp, bool w>() -> gconn_status {
         if constexpr (l != LK_JTB) {   // (Union-JTB keeps no parents in P)
-            if (!sampled && n >= (1u << 18)) {
+            if (dense != never) {
                 auto ka = k_finish_all<l, f, sp, w, OffT>;
-                return launch_pdl("finish", ka, grid_for(ka, B, (uint64_t)n * 32), B, 0, st, off, cols, s,
+                GC_TRY(launch_pdl("finish", ka, grid_for(ka, B, (uint64_t)n * 32), B, 0, st, off, cols, s,
                                   (const uint32_t*)small, (const uint32_t*)(cnt + 0), (const unsigned long long*)tasks,
                                   (const uint32_t*)(cnt + 1), (uint32_t)task_cap, (const uint32_t*)over,
-                                  (const uint32_t*)(cnt + 2));
+                                  (const uint32_t*)(cnt + 2), dense));
+                if (!dense) return GCONN_OK;
             }
         }
         auto k = k_finish<l, f, sp, w, OffT>;
         return launch_pdl("finish", k, grid_for(k, B, (uint64_t)n * 32), B, 0, st, off, cols, s,
                       (const uint32_t*)active, (const uint32_t*)small, (const uint32_t*)(cnt + 0),
                       (const unsigned long long*)tasks, (const uint32_t*)(cnt + 1), (uint32_t)task_cap,
-                      (const uint32_t*)over, (const uint32_t*)(cnt + 2));
+                      (const uint32_t*)over, (const uint32_t*)(cnt + 2), dense == never ? 0 : dense);
     }));
     if (finalized && !jtb) {   // the lists are freed with this call's scratch: finalise now
         GC_TRY(launch_pdl("finalize", k_finalize_gathered, grid_for(k_finalize_gathered, 256, n), 256, 0, st, s,

@@ -1005,13 +1005,17 @@ __device__ __forceinline__ void finish_pass(const OffT* __restrict__ off, const 
     }
 }
 
+// An unsampled pass whose arc count the host does not know launches k_finish and
+// k_finish_all, and the arc count on the device says which of them works: the
+// former below `dense` arcs (0: always), the latter from there.
 template <int L, int F, int S, bool SF, class OffT = uint64_t>
 __global__ void __launch_bounds__(256) k_finish(const OffT* __restrict__ off, const uint32_t* __restrict__ cols,
                                                UFState s, const uint32_t* active, const uint32_t* small,
                                                const uint32_t* nsmall, const unsigned long long* tasks,
                                                const uint32_t* ntasks, uint32_t task_cap, const uint32_t* over,
-                                               const uint32_t* nover) {
+                                               const uint32_t* nover, uint64_t dense) {
     pdl_entry();
+    if (dense && off[s.n] >= dense) return;
     uint32_t ct = *ntasks;
     if (ct > task_cap) ct = task_cap;
     finish_pass<L, F, S, SF, OffT, false>(off, cols, s, active, small, *nsmall, tasks, ct, over, *nover);
@@ -1024,17 +1028,18 @@ __global__ void __launch_bounds__(256) k_finish(const OffT* __restrict__ off, co
 // one gather an edge, the row's own parent is read once).  A list of at least 16
 // vertices a warp is compared and queued too.  RMAT without sampling: n = 2^20,
 // m = 2^24 266 -> 188 us a pass, Union-Async 960 -> 558; n = 2^22, m = 2^26
-// 831 -> 528 (716 with 40 registers a thread, which spill).  Below 2^18 vertices
-// the unions contend and comparing first only delays them (ER n = 16,384,
-// m = 65,536: 60 -> 66 us): k_finish.  After sampling nearly every listed arc joins two trees and the
-// lists are short: k_finish (there the compared parents and the extra registers
-// cost 53 -> 67 us on grid + paths of 8.4 M vertices).
+// 831 -> 528 (716 with 40 registers a thread, which spill).  After sampling nearly
+// every listed arc joins two trees and the lists are short: k_finish (there the
+// compared parents and the extra registers cost 53 -> 67 us on grid + paths of
+// 8.4 M vertices).
 template <int L, int F, int S, bool SF, class OffT = uint64_t>
 __global__ void __launch_bounds__(256, 5) k_finish_all(const OffT* __restrict__ off, const uint32_t* __restrict__ cols,
                                                     UFState s, const uint32_t* small, const uint32_t* nsmall,
                                                     const unsigned long long* tasks, const uint32_t* ntasks,
-                                                    uint32_t task_cap, const uint32_t* over, const uint32_t* nover) {
+                                                    uint32_t task_cap, const uint32_t* over, const uint32_t* nover,
+                                                    uint64_t dense) {
     pdl_entry();
+    if (off[s.n] < dense) return;
     __shared__ QueueSmem<SF> qm;
     UnionQueue<L, F, S, SF> q(s, qm);
     uint32_t ct = *ntasks;

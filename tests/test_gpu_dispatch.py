@@ -107,3 +107,53 @@ def test_coo_forests_around_the_lines(n, m):
         ids, _ = g.spanning_forest(n, dev(e), g.make_variant(link=link, find=find, splice=splice))
         g.gconn_sync()
         assert oracle.sf_check(n, e, ids.cpu().numpy().astype(np.uint64), ref) == 0
+
+
+def _csr_call(n, off, cols, v, bits):
+    import torch
+    lab = torch.empty(n, dtype=torch.int32, device="cuda")
+    f = g.gconn_cc_csr32 if bits == 32 else g.gconn_cc_csr
+    f(n, off, cols, lab, v)
+    g.gconn_sync()
+    return host_u32(lab)
+
+
+@pytest.mark.parametrize("link", ["remcas", "async", "early", "hooks"])
+@pytest.mark.parametrize("n,m,direct", [((1 << 18) - 1, 1 << 21, 1), (1 << 18, 1 << 18, 2), (1 << 18, 1 << 20, 2),
+                                        (1 << 18, (1 << 21) - 1, 2), (1 << 18, 1 << 21, 2), (1 << 20, 1 << 18, 1)])
+def test_unsampled_csr_finish_lines(link, n, m, direct):
+    """A direct call between 2^18 and 2^20 vertices leaves the choice to the arc count on the device, a plan and all
+    other sizes launch the one kernel; the labels are the oracle's either way, also when a plan's contents turn from
+    a sparse graph to a dense one."""
+    import torch
+    g.build()
+    e = graphgen.er(n, m, n + m)
+    off, cols = graphgen.csr(n, e)
+    ref = oracle.cc_uf(n, e)
+    v = g.make_variant(link=link, splice="split_one" if link == "remcas" else "none")
+    assert (_csr_call(n, dev(off), dev(cols), v, 64) == ref).all()
+    assert (_csr_call(n, dev(off.astype(np.uint32)), dev(cols), v, 32) == ref).all()
+    d_off, lab = dev(off.astype(np.uint32)), torch.empty(n, dtype=torch.int32, device="cuda")
+    d_cols = torch.zeros(max(len(cols), 1 << 22), dtype=torch.int32, device="cuda")
+    d_cols[:len(cols)].copy_(dev(cols))
+    g.gconn_profile_enable(True)
+    try:
+        g.gconn_profile_sync()
+        g.gconn_profile_reset()
+        g.gconn_cc_csr32(n, d_off, d_cols, lab, v)
+        g.gconn_profile_sync()
+        assert g.gconn_profile_get()["finish"][0] == direct
+    finally:
+        g.gconn_profile_enable(False)
+    p = g.gconn_plan_create_cc_csr32(n, d_off, d_cols, lab, v)
+    g.gconn_plan_run(p)
+    g.gconn_sync()
+    assert (host_u32(lab) == ref).all()
+    e2 = graphgen.er(n, 1 << 21 if m < 1 << 20 else 1 << 17, 5)
+    o2, c2 = graphgen.csr(n, e2)
+    d_off.copy_(dev(o2.astype(np.uint32)))
+    d_cols[:len(c2)].copy_(dev(c2))
+    g.gconn_plan_run(p)
+    g.gconn_sync()
+    assert (host_u32(lab) == oracle.cc_uf(n, e2)).all()
+    g.gconn_plan_destroy(p)
