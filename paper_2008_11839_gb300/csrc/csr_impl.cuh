@@ -112,7 +112,7 @@ gconn_status csr_sample(const Variant& v, const UFState& s, const OffT* off, con
         JobQueue dq{qbuf.as<KoutJob>(), dq_count, qcap};   // count zeroed by the init kernel
         return dispatch_uf(L, F, S, sf, [&]<int l, int f, int sp, bool w>() {
             auto k = k_hb2w<l, f, sp, w, OffT>;
-            if constexpr (rule_is_bare<l, f>())
+            if constexpr (rule_is_bare<l, f>() && l != LK_HOOKS)
                 if (n >= HB_LONG_N) k = k_hb2w<l, f, sp, w, OffT, HB_LONG_STEPS>;
             GC_TRY(launch_pdl("hb2", k, grid_for(k, 256, n), 256, 0, st, off, cols, v.hb_n, s, dq));
             auto kj = k_union_jobs<l, f, sp, w>;

@@ -226,11 +226,12 @@ struct KoutJob {
 // compression happened) and re-run later from its endpoints by
 // k_union_jobs, so a few long climbs do not hold 31 idle lanes.
 constexpr uint32_t KOUT_FAST_STEPS = 8;
-// HB's second step under rules that compress nothing on the way (naive finds),
-// from HB_LONG_N vertices: there the walks are long whoever runs them, and a
-// deferred union only starts again.  RMAT n = 10^6, Union-Async: 8 steps 110 us a
-// pass, 16 97, 20 95, 32 97; ER n = 2^20 224 -> 200.  Fewer vertices contend and
-// gain from deferral (ER n = 65,536: 60 -> 65), and so do the rules that compress
+// HB's second step under Union-Async with naive finds and Afforest, from
+// HB_LONG_N vertices: there the walks are long whoever runs them, and a deferred
+// union only starts again.  RMAT n = 10^6, Union-Async: 8 steps 110 us a pass, 16 97,
+// 20 95, 32 97; ER n = 2^20, m = 2n 249 -> 219, 8n 134 -> 144.  Fewer vertices contend
+// and gain from deferral (ER n = 65,536: 60 -> 65), and so do Union-Hooks (ER n = 2^20,
+// m = 8n 229 -> 317, n = 2^19, m = 4n 237 -> 270), the rules that compress
 // (Union-Rem-CAS on ER n = 2^20: 85 -> 100) and k-out (RMAT n = 2^22: no gain, ER
 // n = 2^20: 81 -> 98).
 // The budget is a template argument: as a run-time value it costs the default
