@@ -29,7 +29,7 @@ static __global__ void __launch_bounds__(1024, 1) k_small_cc(uint32_t n, const u
 // -> one block):
 // - Rem-CAS climbs one step a turn with full lanes: n = 1,000, m = 4,000 16 -> 8,
 //   m = 64,000 27 -> 18; n = 16,384, m = 32,768 36 -> 30 (ER), 22 -> 18 (RMAT),
-//   m = 65,536 43 -> 36, 33 -> 25; m = 128,000 no gain.
+//   m = 65,536 47 -> 36, 24 -> 25; m = 128,000 no gain.
 // - Union-Async runs a whole union per lane, so a turn takes as long as its longest
 //   walk.  Halving keeps the walks short: n = 4,096, m = 4,096 21 -> 13, m = 65,536
 //   37 -> 28; but n = 16,384, m = 32,768 29 -> 41.  Naive walks grow with the

@@ -229,7 +229,9 @@ constexpr uint32_t KOUT_FAST_STEPS = 8;
 // HB's second step under Union-Async with naive finds and Afforest, from
 // HB_LONG_N vertices: there the walks are long whoever runs them, and a deferred
 // union only starts again.  RMAT n = 10^6, Union-Async: 8 steps 110 us a pass, 16 97,
-// 20 95, 32 97; ER n = 2^20, m = 2n 249 -> 219, 8n 134 -> 144.  Fewer vertices contend
+// 20 95, 32 97; ER n = 2^20, m = 2n 249 -> 219, n = 2^22, m = 4n 531 -> 329.  (Dense ER
+// lists of up to 2^21 vertices lose: n = 2^20, m = 8n 131 -> 141, 16n 139 -> 157; what kind
+// of graph it is the host cannot know.)  Fewer vertices contend
 // and gain from deferral (ER n = 65,536: 60 -> 65), and so do Union-Hooks (ER n = 2^20,
 // m = 8n 229 -> 317, n = 2^19, m = 4n 237 -> 270), the rules that compress
 // (Union-Rem-CAS on ER n = 2^20: 85 -> 100) and k-out (RMAT n = 2^22: no gain, ER
