@@ -260,18 +260,25 @@ gconn_status csr_connect(const Variant& v, const UFState& s, const OffT* off, co
     int L, F, S;
     uf_triple(v, &L, &F, &S);
     int B = block_of(v);
-    // Without sampling the compared-and-queued finish: from 2^20 vertices on any
-    // list (ER, m = n/2 to 16n, RMAT and grids, every rule: 0.34 to 1.1 of the pass
-    // with k_finish), from 2^18 on lists of at least 16 arcs a vertex (Union-Async 8,
-    // Early 32), where fewer edges link (Rem-CAS, ER n = 2^18: m = 2n 94 -> 99 us, 4n
-    // 108 -> 122, 8n 133 -> 128, 16n 195 -> 129; Union-Async n = 2^19: m = n 98 -> 102, 4n
-    // 251 -> 171; Early n = 2^18: 8n 104 -> 113, 16n 162 -> 138).  Below 2^18 the unions
-    // contend and comparing first only delays them (ER n = 2^17, m = 4n, Early:
-    // 71 -> 87).  Where the device makes the choice, the kernel that does not work
-    // costs about 1.3 us of a pass of 33 us and more.
+    // Without sampling the compared-and-queued finish, by vertices and arcs:
+    // - from 2^20 vertices Union-Async, Union-Hooks and Early with compressing finds
+    //   on any list (ER m = n/2 to 16n, RMAT, grids: 0.34 to 1.05 of the pass with
+    //   k_finish), the other rules on lists of at least 4 arcs a vertex (0.64 to
+    //   1.04); below most edges link (grid + paths of 4.2 M vertices, Rem-CAS 829
+    //   -> 885 us, Rem-Lock 1,162 -> 1,300, of 33.5 M Early 2,400 -> 2,566, Afforest 14,710
+    //   -> 16,316).
+    // - from 2^18 on lists of at least 16 arcs a vertex (Union-Async 8, Early 32):
+    //   Rem-CAS, ER n = 2^18: m = 2n 94 -> 99 us, 4n 108 -> 122, 8n 133 -> 128, 16n 195 ->
+    //   129; Union-Async n = 2^19: m = n 98 -> 102, 4n 251 -> 171; Early n = 2^18: 8n 104 ->
+    //   113, 16n 162 -> 138.
+    // - Below 2^18 the unions contend and comparing first only delays them (ER
+    //   n = 2^17, m = 4n, Early: 71 -> 87).
+    // Where the device makes the choice, the kernel that does not work costs about
+    // 1.3 us of a pass of 33 us and more.
     const uint64_t never = UINT64_MAX;
+    const bool walks = L == LK_ASYNC || L == LK_HOOKS || (L == LK_EARLY && F != FD_NAIVE);
     uint64_t dense = sampled || jtb || n < (1u << 18) ? never
-                   : n >= (1u << 20) ? 0 : (uint64_t)n * (L == LK_ASYNC ? 8 : L == LK_EARLY ? 32 : 16);
+                   : (uint64_t)n * (n >= (1u << 20) ? (walks ? 0 : 4) : L == LK_ASYNC ? 8 : L == LK_EARLY ? 32 : 16);
     if (dense && dense != never && csr_arcs_hint() != UINT64_MAX) dense = csr_arcs_hint() >= dense ? 0 : never;
     GC_TRY(dispatch_uf(L, F, S, s.sf != nullptr, [&]<int l, int f, int sp, bool w>() -> gconn_status {
         if constexpr (l != LK_JTB) {   // (Union-JTB keeps no parents in P)

@@ -119,14 +119,15 @@ def _csr_call(n, off, cols, v, bits):
 
 
 @pytest.mark.parametrize("link", ["remcas", "async", "early", "hooks"])
-@pytest.mark.parametrize("n,m,direct", [((1 << 18) - 1, 1 << 21, 1), (1 << 18, 1 << 18, 2), (1 << 18, 1 << 20, 2),
-                                        (1 << 18, (1 << 21) - 1, 2), (1 << 18, 1 << 21, 2), (1 << 20, 1 << 18, 1)])
-def test_unsampled_csr_finish_lines(link, n, m, direct):
-    """A direct call between 2^18 and 2^20 vertices leaves the choice to the arc count on the device, a plan and all
-    other sizes launch the one kernel; the labels are the oracle's either way, also when a plan's contents turn from
-    a sparse graph to a dense one."""
+@pytest.mark.parametrize("n,m", [((1 << 18) - 1, 1 << 21), (1 << 18, 1 << 18), (1 << 18, 1 << 20), (1 << 18, (1 << 21) - 1),
+                                 (1 << 18, 1 << 21), (1 << 20, 1 << 18), (1 << 20, (1 << 21) - 1), (1 << 20, 1 << 21)])
+def test_unsampled_csr_finish_lines(link, n, m):
+    """A direct call between 2^18 and 2^20 vertices, and under Rem and Early with naive finds above, leaves the choice to
+    the arc count on the device; a plan and all other calls launch the one kernel.  The labels are the oracle's either
+    way, also when a plan's contents turn from a sparse graph to a dense one."""
     import torch
     g.build()
+    direct = 1 if n < 1 << 18 or (n >= 1 << 20 and link in ("async", "hooks")) else 2
     e = graphgen.er(n, m, n + m)
     off, cols = graphgen.csr(n, e)
     ref = oracle.cc_uf(n, e)
