@@ -362,8 +362,10 @@ gconn_status gconn_plan_destroy(gconn_plan* p);
  * and edges [edge_off[g], edge_off[g+1]) of the concatenated arrays; its
  * edges use LOCAL ids in [0, n_g) and its labels are LOCAL min ids.
  * Graphs with n_g <= class_max_n[last] run entirely in shared memory (32-bit
- * parents where the class's graphs fit that way (n_g <= 52,976), 16-bit above, one CTA per graph, one persistent kernel per size class on its own
- * stream); larger graphs use the global-memory path one launch each.
+ * parents where the class's largest graph and the warps' queues, 20 bytes a
+ * thread, fit a block that way: n_g <= 52,976 with 1,024 threads, 57,936 with
+ * 32; 16-bit above; one CTA per graph, one persistent kernel per size class on
+ * its own stream); larger graphs use the global-memory path one launch each.
  *   vtx_off, edge_off : uint64[G+1] (device or host; read on the host once)
  *   edges             : uint32[2 * edge_off[G]] pairs, DEVICE memory
  *   labels            : uint32[vtx_off[G]] output, DEVICE memory

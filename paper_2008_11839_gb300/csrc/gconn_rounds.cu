@@ -16,7 +16,7 @@
 //
 // What bounded the rounds: every edge's message was an atomic, and most aim at a
 // few roots; RMAT n = 2^20, m = 2^24 on one GB300, SV / Liu-Tarjan PRF:
-// 1,292 / 5,260 us at first; no atomic for a message that cannot win, finished
+// 1,292 / 4,062-6,067 us at first; no atomic for a message that cannot win, finished
 // edges left out of later rounds (for_live_edges) 605 / 1,034; what a block has
 // sent already remembered in shared memory (SentTable), labels read through L1
 // 375 / 696; compression walks through L1 350 / 629.  1024 x 1024 grid + 16
