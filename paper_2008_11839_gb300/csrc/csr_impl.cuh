@@ -185,6 +185,26 @@ static __global__ void k_sample_stats(const OffT* __restrict__ off, const uint32
     atomicAdd(c + 5, insp);
 }
 
+// Without sampling: the arcs a vertex from which the compared-and-queued finish
+// (k_finish_all) is the faster one, for n >= 2^18; below that many vertices the
+// unions contend and comparing first only delays them (ER n = 2^17, m = 4n, Early:
+// 71 -> 87 us).  From 2^20 vertices Union-Async, Union-Hooks and Early with
+// compressing finds take it on any list (ER m = n/2 to 16n, RMAT, grids: 0.34 to
+// 1.05 of the pass with k_finish), the others where not most edges link (grid +
+// paths of 4.2 M vertices, Rem-CAS 829 -> 885 us, Rem-Lock 1,162 -> 1,300; of 33.5 M, Early
+// 2,400 -> 2,566, Afforest 14,710 -> 16,316).  Between, by ER lists, the kind that
+// gains less (RMAT n = 2^18, m = 2n gains 3 to 24 %): n = 2^18, Rem-CAS m = 2n 94 -> 99, 4n
+// 108 -> 122, 8n 133 -> 128, 16n 195 -> 129, Union-Async 2n 102 -> 113, 4n 165 -> 150, Early 8n
+// 104 -> 113, 16n 162 -> 138, Union-Hooks 2n 312 -> 318, 4n 639 -> 556; n = 2^19, Union-Async n 98 -> 102, 2n 152 -> 126, Afforest 2n 90
+// -> 84, Early with halving 2n 107 -> 108, 4n 132 -> 128, Rem-CAS 4n 109 -> 111, 8n 147 -> 141.
+inline uint64_t dense_arcs(int L, int F, uint32_t n) {
+    const bool async = L == LK_ASYNC, early_find = L == LK_EARLY && F != FD_NAIVE;
+    if (n >= (1u << 20)) return async || L == LK_HOOKS || early_find ? 0 : 4;
+    if (L == LK_HOOKS) return 4;
+    if (n >= (1u << 19)) return async || L == LK_AFFOREST ? 4 : early_find ? 8 : 16;
+    return async ? 8 : L == LK_EARLY ? 32 : 16;
+}
+
 // With `finalized` non-null, a union-find finish also finalises the labels in
 // P (from the gathered lists, k_finalize_gathered) and sets *finalized.
 template <class OffT>
@@ -197,7 +217,8 @@ gconn_status csr_connect(const Variant& v, const UFState& s, const OffT* off, co
     // the pass's counters in one 64-byte header, cleared by the init kernel:
     // [0] L_max, [1..3] gathering counters, [4] the samples' mode label,
     // [8..9] deferred-union count (u64), [10] blocks of the retry kernel done
-    // (the last one resolves L_max)
+    // (the last one resolves L_max), [12..14] lengths that k_finish_all leaves to
+    // k_finish
     GC_TRY(sc.counters.alloc(16 * sizeof(uint32_t), st));
     uint32_t* hdr = sc.counters.as<uint32_t>();
     uint32_t* lmax = sampled ? hdr : nullptr;
@@ -260,26 +281,13 @@ gconn_status csr_connect(const Variant& v, const UFState& s, const OffT* off, co
     int L, F, S;
     uf_triple(v, &L, &F, &S);
     int B = block_of(v);
-    // Without sampling the compared-and-queued finish, by vertices and arcs:
-    // - from 2^20 vertices Union-Async, Union-Hooks and Early with compressing finds
-    //   on any list (ER m = n/2 to 16n, RMAT, grids: 0.34 to 1.05 of the pass with
-    //   k_finish), the other rules on lists of at least 4 arcs a vertex (0.64 to
-    //   1.04); below most edges link (grid + paths of 4.2 M vertices, Rem-CAS 829
-    //   -> 885 us, Rem-Lock 1,162 -> 1,300, of 33.5 M Early 2,400 -> 2,566, Afforest 14,710
-    //   -> 16,316).
-    // - from 2^18 on lists of at least 16 arcs a vertex (Union-Async 8, Early 32):
-    //   Rem-CAS, ER n = 2^18: m = 2n 94 -> 99 us, 4n 108 -> 122, 8n 133 -> 128, 16n 195 ->
-    //   129; Union-Async n = 2^19: m = n 98 -> 102, 4n 251 -> 171; Early n = 2^18: 8n 104 ->
-    //   113, 16n 162 -> 138.
-    // - Below 2^18 the unions contend and comparing first only delays them (ER
-    //   n = 2^17, m = 4n, Early: 71 -> 87).
-    // Where the device makes the choice, the kernel that does not work costs about
-    // 1.3 us of a pass of 33 us and more.
     const uint64_t never = UINT64_MAX;
-    const bool walks = L == LK_ASYNC || L == LK_HOOKS || (L == LK_EARLY && F != FD_NAIVE);
-    uint64_t dense = sampled || jtb || n < (1u << 18) ? never
-                   : (uint64_t)n * (n >= (1u << 20) ? (walks ? 0 : 4) : L == LK_ASYNC ? 8 : L == LK_EARLY ? 32 : 16);
+    uint64_t dense = sampled || jtb || n < (1u << 18) ? never : (uint64_t)n * dense_arcs(L, F, n);
+    // (known on the host for a plan; else the device makes the choice, and the kernel
+    // that does not work costs about 1.3 us of a pass of 33 us and more)
     if (dense && dense != never && csr_arcs_hint() != UINT64_MAX) dense = csr_arcs_hint() >= dense ? 0 : never;
+    uint32_t* next = hdr + 12;
+    const uint32_t* len = cnt;   // the lists' lengths for k_finish
     GC_TRY(dispatch_uf(L, F, S, s.sf != nullptr, [&]<int l, int f, int sp, bool w>() -> gconn_status {
         if constexpr (l != LK_JTB) {   // (Union-JTB keeps no parents in P)
             if (dense != never) {
@@ -287,15 +295,15 @@ gconn_status csr_connect(const Variant& v, const UFState& s, const OffT* off, co
                 GC_TRY(launch_pdl("finish", ka, grid_for(ka, B, (uint64_t)n * 32), B, 0, st, off, cols, s,
                                   (const uint32_t*)small, (const uint32_t*)(cnt + 0), (const unsigned long long*)tasks,
                                   (const uint32_t*)(cnt + 1), (uint32_t)task_cap, (const uint32_t*)over,
-                                  (const uint32_t*)(cnt + 2), dense));
+                                  (const uint32_t*)(cnt + 2), dense, dense ? next : nullptr));
                 if (!dense) return GCONN_OK;
+                len = next;
             }
         }
         auto k = k_finish<l, f, sp, w, OffT>;
         return launch_pdl("finish", k, grid_for(k, B, (uint64_t)n * 32), B, 0, st, off, cols, s,
-                      (const uint32_t*)active, (const uint32_t*)small, (const uint32_t*)(cnt + 0),
-                      (const unsigned long long*)tasks, (const uint32_t*)(cnt + 1), (uint32_t)task_cap,
-                      (const uint32_t*)over, (const uint32_t*)(cnt + 2), dense == never ? 0 : dense);
+                      (const uint32_t*)active, (const uint32_t*)small, len + 0, (const unsigned long long*)tasks,
+                      len + 1, (uint32_t)task_cap, (const uint32_t*)over, len + 2);
     }));
     if (finalized && !jtb) {   // the lists are freed with this call's scratch: finalise now
         GC_TRY(launch_pdl("finalize", k_finalize_gathered, grid_for(k_finalize_gathered, 256, n), 256, 0, st, s,

@@ -1008,17 +1008,13 @@ __device__ __forceinline__ void finish_pass(const OffT* __restrict__ off, const 
     }
 }
 
-// An unsampled pass whose arc count the host does not know launches k_finish and
-// k_finish_all, and the arc count on the device says which of them works: the
-// former below `dense` arcs (0: always), the latter from there.
 template <int L, int F, int S, bool SF, class OffT = uint64_t>
 __global__ void __launch_bounds__(256) k_finish(const OffT* __restrict__ off, const uint32_t* __restrict__ cols,
                                                UFState s, const uint32_t* active, const uint32_t* small,
                                                const uint32_t* nsmall, const unsigned long long* tasks,
                                                const uint32_t* ntasks, uint32_t task_cap, const uint32_t* over,
-                                               const uint32_t* nover, uint64_t dense) {
+                                               const uint32_t* nover) {
     pdl_entry();
-    if (dense && off[s.n] >= dense) return;
     uint32_t ct = *ntasks;
     if (ct > task_cap) ct = task_cap;
     finish_pass<L, F, S, SF, OffT, false>(off, cols, s, active, small, *nsmall, tasks, ct, over, *nover);
@@ -1035,14 +1031,25 @@ __global__ void __launch_bounds__(256) k_finish(const OffT* __restrict__ off, co
 // every listed arc joins two trees and the lists are short: k_finish (there the
 // compared parents and the extra registers cost 53 -> 67 us on grid + paths of
 // 8.4 M vertices).
+// Where the host does not know the arc count (next is given), it does nothing below
+// `dense` arcs, and k_finish follows with the list lengths that block 0 leaves in
+// next: none if this kernel worked, else the lists'.
 template <int L, int F, int S, bool SF, class OffT = uint64_t>
 __global__ void __launch_bounds__(256, 5) k_finish_all(const OffT* __restrict__ off, const uint32_t* __restrict__ cols,
                                                     UFState s, const uint32_t* small, const uint32_t* nsmall,
                                                     const unsigned long long* tasks, const uint32_t* ntasks,
                                                     uint32_t task_cap, const uint32_t* over, const uint32_t* nover,
-                                                    uint64_t dense) {
+                                                    uint64_t dense, uint32_t* next) {
     pdl_entry();
-    if (off[s.n] < dense) return;
+    if (next) {
+        const bool mine = off[s.n] >= dense;
+        if (blockIdx.x == 0 && threadIdx.x == 0) {
+            next[0] = mine ? 0u : *nsmall;
+            next[1] = mine ? 0u : *ntasks;
+            next[2] = mine ? 0u : *nover;
+        }
+        if (!mine) return;
+    }
     __shared__ QueueSmem<SF> qm;
     UnionQueue<L, F, S, SF> q(s, qm);
     uint32_t ct = *ntasks;
