@@ -30,16 +30,18 @@ constexpr int NCLS = GCONN_BATCH_CLASSES;
 constexpr uint32_t SMEM_MAX_N = 65536;
 // The form of a class's kernel, by its edges per thread of a block (mean over the
 // class).  Eight rows of edges at a time cost 64 registers a thread, so half the
-// blocks of a small class are resident: from 64 edges a thread the loads in
-// flight are worth it.  Below, two rows a turn (31 registers), and below 4 edges a
-// thread its own unions without the queue (24).  Microseconds a batch, one union
-// per thread / eight rows / two rows / direct: 8,192 graphs of 128 to 1,024
-// vertices, m = n 55 / 80 / 59 / 53 (2.2 edges a thread), m = 4n 95 / 109 / 86 / 95
-// (9); 65,536 graphs of 8 to 32 vertices 124 / 286 / 154 / 127; 4,096 graphs of 1,000
-// to 4,096, m = 12n 268 / 268 / 265 / 367 (120); 300 graphs of 16,384 to 50,000, m = 4n
-// 207 / 159 / 178 / 275 (518).  Blocks of one warp lose no resident block to the
-// registers and keep eight rows (m = 16n on 32 to 128 vertices, 40 edges a thread:
-// 66 / 49 / 68).
+// blocks of a small class are resident: where graphs wait for a block, the loads in
+// flight are worth it from 64 edges a thread.  Below, two rows a turn (31 registers),
+// and below 4 edges a thread its own unions without the queue (24).  Microseconds a
+// batch, one union per thread / eight rows / two rows / direct: 8,192 graphs of 128
+// to 1,024 vertices, m = n 55 / 80 / 59 / 53 (2.2 edges a thread), m = 4n 95 / 109 / 86 /
+// 95 (9); 65,536 graphs of 8 to 32 vertices 124 / 286 / 154 / 127; 4,096 graphs of 1,000 to
+// 4,096, m = 12n 268 / 268 / 265 / 367 (120); 300 graphs of 16,384 to 50,000, m = 4n
+// 207 / 159 / 178 / 275 (518).  Where no graph waits (at most 608 blocks of 256
+// threads) eight rows are the shortest way from a single edge a thread (eight / two /
+// direct: 300 graphs of 1,025 to 2,600, m = 12n 33 / 52 / 91; 550 to 1,000, m = 4n 12 / 13 / 18;
+// 100 of 20 to 100 8 / 8 / 7).  Blocks of one warp lose no resident block to the registers
+// and keep eight rows (m = 16n on 32 to 128 vertices, 40 edges a thread: 66 / 49 / 68).
 constexpr uint64_t BATCH_FULL = 64, BATCH_LEAN = 4;
 
 // Persistent class kernel: CTAs pull graph indices (largest first) from an
@@ -115,15 +117,21 @@ static gconn_status launch_class(gconn_batch* b, int c, int block, int rule, cud
     if (!cnt) return GCONN_OK;
     const bool wide = smem_wide(b->cls_maxn[c], block);   // 32-bit parents (no 16-bit CAS)
     const size_t smem = smem_cc_bytes(b->cls_maxn[c], block);
-    const uint64_t threads = (uint64_t)block * cnt, m = b->cls_edges[c];
-    const BatchKernel k = !wide ? rule_kernel<uint16_t, BATCH_ILP>(rule)
-                        : block == 32 || m >= BATCH_FULL * threads ? rule_kernel<uint32_t, BATCH_ILP>(rule)
-                        : m >= BATCH_LEAN * threads ? rule_kernel<uint32_t, 2>(rule) : rule_kernel<uint32_t, 1>(rule);
     int per_sm = 0;
-    // always the largest block's size: plans made by several threads share the attribute
-    GC_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BLOCK_MAX));
-    GC_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, block, smem));
-    if (per_sm < 1) return GCONN_E_UNSUPPORTED;
+    auto occupancy = [&](BatchKernel k) -> gconn_status {
+        // always the largest block's size: plans made by several threads share the attribute
+        GC_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BLOCK_MAX));
+        GC_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, block, smem));
+        return per_sm < 1 ? GCONN_E_UNSUPPORTED : GCONN_OK;
+    };
+    BatchKernel k = wide ? rule_kernel<uint32_t, BATCH_ILP>(rule) : rule_kernel<uint16_t, BATCH_ILP>(rule);
+    GC_TRY(occupancy(k));
+    const uint64_t threads = (uint64_t)block * cnt, m = b->cls_edges[c];
+    const bool waits = cnt > (uint64_t)per_sm * num_sms();   // more graphs than resident blocks
+    if (wide && block > 32 && (m < threads || (waits && m < BATCH_FULL * threads))) {
+        k = m < (waits ? BATCH_LEAN : 1) * threads ? rule_kernel<uint32_t, 1>(rule) : rule_kernel<uint32_t, 2>(rule);
+        GC_TRY(occupancy(k));
+    }
     uint32_t grid = (uint32_t)std::min<uint64_t>((uint64_t)per_sm * num_sms(), cnt);
     return launch("batch_smem", k, grid, block, smem, st, b->vo, b->eo, (const uint2*)b->edges, b->labels,
                   b->order + b->cls_begin[c], cnt, b->queues + c, err_word());

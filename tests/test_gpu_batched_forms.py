@@ -29,11 +29,15 @@ def _run(graphs, block, rule):
 @pytest.mark.parametrize("rule", [("async", "naive"), ("async", "halve"), ("remcas", "naive")])
 @pytest.mark.parametrize("block", [32, 64, 256, 1024])
 def test_mean_edges_around_the_lines(block, rule):
-    """One class: every graph with the same edge count, just below, at and above 4 and 64 a thread."""
+    """One class: every graph with the same edge count, just below, at and above 1, 4 and 64 a thread, as a few graphs
+    and (short lists only) as more graphs than blocks are resident."""
     g.build()
-    for per in (4, 64):
+    for per in (1, 4, 64):
         for m in (per * block - 1, per * block, per * block + 33):
             _run([(701 + k, graphgen.er(701 + k, m, m + k)) for k in range(5)], block, rule)
+            if m <= 20000 and block > 32:
+                base = [(701 + k, graphgen.er(701 + k, m, m + k)) for k in range(3)]
+                _run(base * (max(2600 // (block // 32), 200)), block, rule)
 
 
 @pytest.mark.parametrize("block", [32, 256, 1024])
